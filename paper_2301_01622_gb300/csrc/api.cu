@@ -329,11 +329,12 @@ int llb_create(llb_ctx** out, int nx, int ny, int nz, int lattice, double tau, c
     }
     c->diag_scratch_bytes = (size_t)diag_blocks(*c) * 16 * sizeof(double) + 256;
     if (cudaMalloc(&c->diag_scratch, c->diag_scratch_bytes + sizeof(llb_diag)) != cudaSuccess) { cudaGetLastError(); c->diag_scratch = nullptr; return bail(LLB_ENOMEM); }
-    if (cudaMalloc(&c->flag_dev, 2 * sizeof(int)) != cudaSuccess) { cudaGetLastError(); c->flag_dev = nullptr; return bail(LLB_ENOMEM); }
+    if (cudaMalloc(&c->flag_dev, 4 * sizeof(int)) != cudaSuccess) { cudaGetLastError(); c->flag_dev = nullptr; return bail(LLB_ENOMEM); }
     c->err_dev = static_cast<int*>(c->flag_dev) + 1;
+    c->queue_dev = static_cast<int*>(c->flag_dev) + 2;
     if (c->scheme != LLB_SCHEME_MOMENT && c->ncomp == 2 &&
         cudaMalloc(&c->phi_scratch, c->N * c->elem) != cudaSuccess) { cudaGetLastError(); c->phi_scratch = nullptr; return bail(LLB_ENOMEM); }
-    if (cudaMemsetAsync(c->flag_dev, 0, 2 * sizeof(int), c->stream) != cudaSuccess) { cudaGetLastError(); return bail(LLB_ECUDA); }
+    if (cudaMemsetAsync(c->flag_dev, 0, 4 * sizeof(int), c->stream) != cudaSuccess) { cudaGetLastError(); return bail(LLB_ECUDA); }
     if (c->scheme == LLB_SCHEME_MOMENT && c->ncomp == 2) {
         c->tile_ctas = cg_tiled_ctas(*c);
         cudaGetLastError();

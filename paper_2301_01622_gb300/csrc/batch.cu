@@ -19,6 +19,7 @@ struct llb_batch {
     int n = 0;
     std::vector<llb_ctx*> ctx;
     llb::BatchDom* dev_doms[2] = {nullptr, nullptr};
+    llb::CgMaps* dev_maps[2] = {nullptr, nullptr};  // tensor maps of the boxes (FP32 state)
     int* dev_next = nullptr;  // work queue: next item to take (zeroed before every launch)
     int total = 0;   // work items over all boxes
     int grid = 0;    // persistent CTAs
@@ -48,6 +49,10 @@ int build_tables(llb_batch* b) {
     std::vector<llb::BatchDom> h[2];
     h[0].resize(b->n);
     h[1].resize(b->n);
+    const bool with_maps = b->ctx[0]->storage == LLB_F32;
+    std::vector<llb::CgMaps> maps[2];
+    maps[0].resize(with_maps ? b->n : 0);
+    maps[1].resize(with_maps ? b->n : 0);
     int begin = 0;
     for (int d = 0; d < b->n; ++d) {
         llb_ctx* c = b->ctx[d];
@@ -59,11 +64,13 @@ int build_tables(llb_batch* b) {
         llb::cg_batch_plan(*c, g, &dom);
         dom.lay = c->lay;
         dom.item_begin = begin;
+        dom.err = static_cast<int*>(c->err_dev);
         begin += dom.nitems;
         for (int k = 0; k < 2; ++k) {
             h[k][d] = dom;
             h[k][d].in = c->buf[k];
             h[k][d].out = c->buf[1 - k];
+            if (with_maps && !llb::cg_batch_maps(*c, c->buf[k], c->buf[1 - k], &maps[k][d])) return LLB_ECUDA;
         }
     }
     if (!b->dev_next && cudaMalloc(&b->dev_next, sizeof(int)) != cudaSuccess) {
@@ -82,6 +89,17 @@ int build_tables(llb_batch* b) {
             cudaGetLastError();
             return LLB_ECUDA;
         }
+        if (!with_maps) continue;
+        if (!b->dev_maps[k] && cudaMalloc(&b->dev_maps[k], sizeof(llb::CgMaps) * b->n) != cudaSuccess) {
+            cudaGetLastError();
+            b->dev_maps[k] = nullptr;
+            return LLB_ENOMEM;
+        }
+        if (cudaMemcpy(b->dev_maps[k], maps[k].data(), sizeof(llb::CgMaps) * b->n, cudaMemcpyHostToDevice) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return LLB_ECUDA;
+        }
     }
     b->total = begin;
     b->grid = grid < begin ? grid : begin;
@@ -92,7 +110,8 @@ int build_tables(llb_batch* b) {
 cudaError_t launch(llb_batch* b, int parity) {
     const cudaError_t e = cudaMemsetAsync(b->dev_next, 0, sizeof(int), b->ctx[0]->stream);
     if (e != cudaSuccess) return e;
-    return llb::launch_cg_batch(*b->ctx[0], b->dev_doms[parity], b->n, b->total, b->grid, b->dev_next);
+    return llb::launch_cg_batch(*b->ctx[0], b->dev_doms[parity], b->dev_maps[parity], b->n, b->total, b->grid,
+                                b->dev_next);
 }
 
 void advance(llb_batch* b, int nsteps) {
@@ -151,6 +170,8 @@ void llb_batch_destroy(llb_batch* b) {
     drop_graphs(b);
     for (int k = 0; k < 2; ++k)
         if (b->dev_doms[k]) cudaFree(b->dev_doms[k]);
+    for (int k = 0; k < 2; ++k)
+        if (b->dev_maps[k]) cudaFree(b->dev_maps[k]);
     if (b->dev_next) cudaFree(b->dev_next);
     for (llb_ctx* c : b->ctx) {
         c->in_batch = false;

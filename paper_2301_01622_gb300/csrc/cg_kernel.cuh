@@ -663,17 +663,24 @@ inline Sched2 plan2(int nx, int ny, int nz, int BX, int BY, int grid) {
 }
 
 // Two-component kernel shapes: tile BX x BY, CTAs per SM, approximate FP32
-// divisions (phi, 1/rho, 1/|G|).  Variant 0 is the default.
+// divisions (phi, 1/rho, 1/|G|).
 template <int BX_, int BY_, int MINB_, bool FAST_, bool ROLLED_ = false>
 struct CGShape {
     static constexpr int BX = BX_, BY = BY_, MINB = MINB_;
     static constexpr bool FAST = FAST_, ROLLED = ROLLED_;
+    static constexpr bool PAIR = false;
+};
+// FP32, variant 0 (the default): two nodes per thread (cg_pair.cuh).  On the 384 x 192 x
+// 192 droplet pair 459 us per step on D3Q27 (30.8 k MLUPS) against 740 us of the best
+// one-node shape, 32 x 8 approximate rolled, whose place it takes.
+struct CGPair {
+    static constexpr bool PAIR = true;
 };
 // The approximate quotients measured 18 % (D3Q27) to 23 % (D3Q19) faster on
 // the 384 x 192 x 192 droplet pair and stay within the FP32 parity bound; the
 // rolled plane loop a further 10 % on D3Q27 (fewer instruction-cache misses)
 // and 1 % slower on D3Q19.
-template <class T, int V> struct CGVariant { using type = CGShape<32, 8, 2, true, true>; };
+template <class T, int V> struct CGVariant { using type = CGPair; };
 template <> struct CGVariant<float, 1> { using type = CGShape<64, 4, 2, false>; };
 template <> struct CGVariant<float, 2> { using type = CGShape<32, 8, 2, false>; };
 template <> struct CGVariant<float, 3> { using type = CGShape<32, 16, 1, false>; };

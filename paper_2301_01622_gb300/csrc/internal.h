@@ -35,6 +35,7 @@ struct llb_ctx {
     CUtensorMap pmap[2];     // TMA L2-prefetch descriptors of buf[0], buf[1] (tiled kernel)
     bool pmap_ok = false;
     void* err_dev = nullptr; // device int: set by a kernel whose bounded wait gave up
+    void* queue_dev = nullptr; // two device ints: work queue of the two-component step, zero between launches
     void* buf[2] = {nullptr, nullptr};
     bool owns[2] = {false, false};
     int cur = 0;             // buf[cur] holds the state at time t
@@ -108,6 +109,14 @@ cudaError_t launch_cg_tiled(const llb_ctx& c, const void* in, void* out);
 // Output planes zlo .. zhi-1 on stream st.
 cudaError_t launch_cg_tiled_range(const llb_ctx& c, const void* in, void* out, int zlo, int zhi, cudaStream_t st);
 
+// Tensor maps of one step of the two-component pair kernel: input boxes of
+// (rho1, d) and of the other nine fields, output box.
+struct CgMaps {
+    CUtensorMap rd, m, out;
+};
+// 4D FP32 tensor map (extents and box in elements, strides of dimensions 1..3 in bytes).
+bool encode_f32_map(void* base, const size_t* dims, const size_t* strides, const int* box, CUtensorMap* out);
+
 // One box of a batched ensemble: its state copies for this step and its items.
 struct BatchDom {
     const void* in;
@@ -115,13 +124,18 @@ struct BatchDom {
     Layout lay;
     int ncx, ntiles, zc, nitems;  // chunk-major schedule of the box
     int item_begin;               // first global item of the box
+    int* err;                     // error word of the box
 };
 // Persistent grid size of the batch kernel (ctx gives lattice, storage, variant).
 int cg_batch_ctas(const llb_ctx& c);
 // Fill the schedule fields of d for box c (c.nx.. give the box size) and `grid` CTAs.
 void cg_batch_plan(const llb_ctx& c, int grid, BatchDom* d);
 // `next`: work-queue counter, zero at launch.
-cudaError_t launch_cg_batch(const llb_ctx& c, const BatchDom* doms, int ndom, int total, int grid, int* next);
+// maps: one entry per box (cg_batch_maps; unused by the variants without tensor maps).
+cudaError_t launch_cg_batch(const llb_ctx& c, const BatchDom* doms, const CgMaps* maps, int ndom, int total, int grid,
+                            int* next);
+// Tensor maps of box c stepping from `in` to `out`; false if they cannot be encoded.
+bool cg_batch_maps(const llb_ctx& c, const void* in, void* out, CgMaps* m);
 
 // Bounds-check records of the kernel translation units (checked build; the
 // normal build reports none).  Read and clear; -1 if the copy fails.

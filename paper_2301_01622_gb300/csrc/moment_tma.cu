@@ -271,19 +271,40 @@ bool tma_encode(const llb_ctx& c, void* buf, CUtensorMap* out) { LLB_TMA_VARIANT
 
 }  // namespace
 
+namespace {
+
+// The driver's tensor-map encoder, looked up once; null if the driver has none.
+PFN_cuTensorMapEncodeTiled_v12000 map_encoder() {
+    static const PFN_cuTensorMapEncodeTiled_v12000 encode = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
+        cudaDriverEntryPointQueryResult q;
+        void* fn = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess || q != cudaDriverEntryPointSuccess)
+            return nullptr;
+        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    }();
+    return encode;
+}
+
+}  // namespace
+
+bool encode_f32_map(void* base, const size_t* dims, const size_t* strides, const int* box, CUtensorMap* out) {
+    const auto encode = map_encoder();
+    if (!encode) return false;
+    const cuuint64_t d[4] = {dims[0], dims[1], dims[2], dims[3]}, s[3] = {strides[0], strides[1], strides[2]};
+    const cuuint32_t b[4] = {(cuuint32_t)box[0], (cuuint32_t)box[1], (cuuint32_t)box[2], (cuuint32_t)box[3]};
+    const cuuint32_t e[4] = {1, 1, 1, 1};
+    return encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, d, s, b, e, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // 4D tensor map (x, y, z, field) of a moment state buffer with a box of
 // box_w x box_h nodes of one plane and all ten fields, element type of the
 // context's storage.  False if the driver entry point or the encoding fails.
 bool encode_box_map(const llb_ctx& c, void* buf, int box_w, int box_h, CUtensorMap* out) {
-    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-    if (!encode) {
-        cudaDriverEntryPointQueryResult q;
-        void* fn = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess || q != cudaDriverEntryPointSuccess || !fn)
-            return false;
-        encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
+    const auto encode = map_encoder();
+    if (!encode) return false;
     const Layout& Lo = c.lay;
     if (!Lo.ghosts || c.ncomp != 1 || box_w > 256 || box_h > 256) return false;
     CUtensorMapDataType dt;
