@@ -49,6 +49,69 @@ namespace {
 
 constexpr int kAdjThreads = 128;
 
+// dL/domega term of a node, lam'_A : (j j / rho - A), and its sums.  In FP64 these
+// some 40 operations per node filled the FP64 pipe (two FMA per clock and SM; 79 %
+// busy) and set the time of the adjoint step, 62 of 62 us on 128 x 96 x 64 D3Q19
+// FP32.  For an FP32 state they run on pairs of FP32 numbers, value = h + l with
+// the rounding error of h in l (exact products by FMA, exact sums by Knuth's
+// two-sum), about 2^-46 relative; FP64 states keep FP64.
+template <class T>
+struct Wide;
+
+template <>
+struct Wide<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double h) { v += h; }
+    // += a (b r - c)
+    __device__ __forceinline__ void add_term(double a, double b, double r, double c) { v += a * (b * r - c); }
+    __device__ __forceinline__ double value() const { return v; }
+    __device__ __forceinline__ Wide shfl_down(int off) const { return {__shfl_down_sync(0xffffffffu, v, off)}; }
+    __device__ __forceinline__ void merge(const Wide& o) { v += o.v; }
+};
+
+template <>
+struct Wide<float> {
+    float h = 0.0f, l = 0.0f;
+    __device__ __forceinline__ void add(float a) {  // two-sum
+        const float s = __fadd_rn(h, a), t = __fsub_rn(s, h);
+        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(a, t)));
+        h = s;
+    }
+    __device__ __forceinline__ void add_term(float a, float b, float r, float c) {
+        const float p = __fmul_rn(b, r), pe = __fmaf_rn(b, r, -p);            // b r = p + pe
+        const float s = __fsub_rn(p, c), t = __fsub_rn(s, p);                 // p - c = s + se
+        const float se = __fsub_rn(__fsub_rn(p, __fsub_rn(s, t)), __fadd_rn(c, t));
+        const float x = __fmul_rn(a, s), xe = __fmaf_rn(a, __fadd_rn(pe, se), __fmaf_rn(a, s, -x));
+        add(x);
+        l = __fadd_rn(l, xe);
+    }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+    __device__ __forceinline__ Wide shfl_down(int off) const {
+        Wide o;
+        o.h = __shfl_down_sync(0xffffffffu, h, off);
+        o.l = __shfl_down_sync(0xffffffffu, l, off);
+        return o;
+    }
+    __device__ __forceinline__ void merge(const Wide& o) {
+        add(o.h);
+        l = __fadd_rn(l, o.l);
+    }
+};
+
+// Sum of the block's terms, added to its row (fixed order: warp shuffles, then the warps).
+template <int NT, class T>
+__device__ __forceinline__ void add_block_sum(Wide<T> part, double* __restrict__ row) {
+    for (int off = 16; off > 0; off >>= 1) part.merge(part.shfl_down(off));
+    __shared__ double wsum[NT / 32];
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = part.value();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double sacc = 0.0;
+        for (int w = 0; w < NT / 32; ++w) sacc += wsum[w];
+        *row += sacc;
+    }
+}
+
 // The ten fields of node i of a one-component buffer (state or cotangent; the
 // field order of FieldMap).
 template <class T>
@@ -66,7 +129,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_step(const T* __restric
                                                               double* __restrict__ domega_rows) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
-    double part = 0.0;
+    Wide<T> part;
     if (x < lay.nx) {
         // lam' = sum_i r_i (e_i . lam_new(y + c_i))
         T ld = T(0), lj[3] = {T(0), T(0), T(0)}, la[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
@@ -117,19 +180,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_step(const T* __restric
 #pragma unroll
         for (int f = 0; f < 10; ++f) lam[FieldMap<T, 10>::at(i0, f, lay.fs)] = out[f];
         // dL/domega: lam'_A : (j j / rho - A)
-        for (int k = 0; k < 6; ++k) part += (double)la[k] * ((double)jj[k] * (double)rinv - (double)s[4 + k]);
+        for (int k = 0; k < 6; ++k) part.add_term(la[k], jj[k], rinv, s[4 + k]);
     }
-    // block sum of the omega derivative (fixed order: warp shuffles then lanes of warp 0)
-    for (int off = 16; off > 0; off >>= 1) part += __shfl_down_sync(0xffffffffu, part, off);
-    __shared__ double wsum[kAdjThreads / 32];
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sacc = 0.0;
-        for (int w = 0; w < kAdjThreads / 32; ++w) sacc += wsum[w];
-        const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        domega_rows[b] = sacc;
-    }
+    add_block_sum<kAdjThreads>(part, domega_rows + ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
 
 template <class T>
@@ -154,7 +207,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_cg_local(const T* __res
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     const size_t fs = lay.fs;
-    double part = 0.0;
+    Wide<T> part;
     if (x < lay.nx) {
         const size_t i0 = lay.at(x, y, z);
         T s[11];
@@ -269,18 +322,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_cg_local(const T* __res
         for (int f = 0; f < 11; ++f) lam[f * fs + i0] = out[f];
 #pragma unroll
         for (int a = 0; a < 3; ++a) lam_g[a * fs + i0] = lg[a];
-        for (int k = 0; k < 6; ++k) part += (double)la[k] * ((double)jj[k] * (double)rinv - (double)A[k]);
+        for (int k = 0; k < 6; ++k) part.add_term(la[k], jj[k], rinv, A[k]);
     }
-    for (int off = 16; off > 0; off >>= 1) part += __shfl_down_sync(0xffffffffu, part, off);
-    __shared__ double wsum[kAdjThreads / 32];
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = part;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sacc = 0.0;
-        for (int w = 0; w < kAdjThreads / 32; ++w) sacc += wsum[w];
-        const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        domega_rows[b] = sacc;
-    }
+    add_block_sum<kAdjThreads>(part, domega_rows + ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
 
 // Pass 2: the phase-field chain at node z.  G(y) = 3 sum_k w_k c_k phi(y + c_k)
@@ -386,13 +430,13 @@ __device__ __forceinline__ void adj_publish(const T* __restrict__ lam_new, const
 
 // Receiver y (node n of the region, own 11 fields in s): the direct kernel's
 // arithmetic with the neighbour quantities read from the ring planes Sm, S0, Sp
-// (planes z - 1, z, z + 1).  Writes lam(y), lam_g(y); returns y's dL/domega term.
+// (planes z - 1, z, z + 1).  Writes lam(y), lam_g(y); adds y's dL/domega term to part.
 template <class L, class T, int HX, int HN>
-__device__ __forceinline__ double adj_receive(const T* __restrict__ Sm, const T* __restrict__ S0,
-                                              const T* __restrict__ Sp, int n, const T* s, const CGAdjPar<T>& p,
-                                              T* __restrict__ lam, T* __restrict__ lam_g, size_t i0, size_t fs) {
+__device__ __forceinline__ void adj_receive(Wide<T>& part, const T* __restrict__ Sm, const T* __restrict__ S0,
+                                            const T* __restrict__ Sp, int n, const T* s, const CGAdjPar<T>& p,
+                                            T* __restrict__ lam, T* __restrict__ lam_g, size_t i0, size_t fs) {
     if (!LLB_IN(n - HX - 1, HN, kChkGather) || !LLB_IN(n + HX + 1, HN, kChkGather) || !LLB_IN(i0, fs, kChkStore))
-        return 0.0;
+        return;
     constexpr int Q = L::Q;
     const T r1 = s[0], d = s[1], jx = s[2], jy = s[3], jz = s[4];
     const T* A = s + 5;  // xx, yy, zz, xy, xz, yz
@@ -489,9 +533,7 @@ __device__ __forceinline__ double adj_receive(const T* __restrict__ Sm, const T*
     for (int f = 0; f < 11; ++f) lam[f * fs + i0] = out[f];
 #pragma unroll
     for (int a = 0; a < 3; ++a) lam_g[a * fs + i0] = ln[a] / gn + l_gn * G[a] / gn;
-    double part = 0.0;
-    for (int k = 0; k < 6; ++k) part += (double)la[k] * ((double)jj[k] * (double)rinv - (double)A[k]);
-    return part;
+    for (int k = 0; k < 6; ++k) part.add_term(la[k], jj[k], rinv, A[k]);
 }
 
 template <class L, class T, int BX, int BY>
@@ -507,7 +549,7 @@ __global__ void __launch_bounds__(BX * BY, (AdjTile<L, T, BX, BY>::MINB))
     const size_t fs = lay.fs, plane = (size_t)lay.px * lay.py;
     const int t = threadIdx.x, tx = t % BX, ty = t / BX;
     const int n_own = (ty + 1) * HX + (tx + 1);
-    double part = 0.0;
+    Wide<T> part;
 
     for (int it = blockIdx.x; it < sc.nitems; it += gridDim.x) {
         int x0, y0, za, zb;  // receivers of planes za .. zb-1 of the tile at (x0, y0)
@@ -537,19 +579,11 @@ __global__ void __launch_bounds__(BX * BY, (AdjTile<L, T, BX, BY>::MINB))
                 for (int f = 0; f < 11; ++f) sv[f] = m[f * fs + iy];
             }
             __syncthreads();  // planes q - 1, q, q + 1 published
-            if (ok) part += adj_receive<L, T, HX, HN>(slot(q - 1), slot(q), slot(q + 1), n_own, sv, p, lam, lam_g, iy, fs);
+            if (ok) adj_receive<L, T, HX, HN>(part, slot(q - 1), slot(q), slot(q + 1), n_own, sv, p, lam, lam_g, iy, fs);
             __syncthreads();  // the slot of plane q - 1 may be refilled
         }
     }
-    for (int off = 16; off > 0; off >>= 1) part += __shfl_down_sync(0xffffffffu, part, off);
-    __shared__ double wsum[NT / 32];
-    if ((t & 31) == 0) wsum[t >> 5] = part;
-    __syncthreads();
-    if (t == 0) {
-        double sacc = 0.0;
-        for (int w = 0; w < NT / 32; ++w) sacc += wsum[w];
-        domega_rows[blockIdx.x] = sacc;
-    }
+    add_block_sum<NT>(part, domega_rows + blockIdx.x);
 }
 
 // acc += sum of rows (one block, fixed order).
@@ -717,14 +751,23 @@ int grid_n(const llb_ctx& c) {
     return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
-// Advance the context by one step (same kernels as llb_step), flipping cur.
+// One forward step (same kernels as llb_step) from `in` to `out`.
+cudaError_t fwd(const llb_ctx& c, const void* in, void* out) {
+    return c.ncomp == 2                   ? launch_cg_tiled(c, in, out)
+           : c.kernel == LLB_KERNEL_TMA   ? launch_moment_tma(c, c.cur, out)
+           : c.kernel == LLB_KERNEL_TILED ? launch_moment_tiled(c, c.cur, in, out)
+                                          : launch_moment_direct(c, in, out);
+}
+
+// Whether fwd takes any pair of state buffers: the TMA-staged kernel and the L2
+// prefetch of tiled variant 1 hold tensor maps of the context's own two buffers.
+bool any_buffer(const llb_ctx& c) {
+    return c.ncomp == 2 || c.kernel == LLB_KERNEL_DIRECT || (c.kernel == LLB_KERNEL_TILED && c.variant != 1);
+}
+
+// Advance the context by one step, flipping cur.
 cudaError_t fwd_one(llb_ctx* c) {
-    const void* in = c->buf[c->cur];
-    void* out = c->buf[1 - c->cur];
-    const cudaError_t e = c->ncomp == 2                   ? launch_cg_tiled(*c, in, out)
-                          : c->kernel == LLB_KERNEL_TMA   ? launch_moment_tma(*c, c->cur, out)
-                          : c->kernel == LLB_KERNEL_TILED ? launch_moment_tiled(*c, c->cur, in, out)
-                                                          : launch_moment_direct(*c, in, out);
+    const cudaError_t e = fwd(*c, c->buf[c->cur], c->buf[1 - c->cur]);
     if (e == cudaSuccess) c->cur = 1 - c->cur;
     return e;
 }
@@ -782,6 +825,7 @@ extern "C" int llb_adjoint(llb_ctx* c, int nsteps, int every, const void* dev_gf
     const int cur0 = c->cur;
     const long long t0 = c->t;
     cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(double), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, nrows * sizeof(double), c->stream);
     // forward with checkpoints (checkpoint k = state at step k K)
     for (int s = 0; s < nsteps && e == cudaSuccess; ++s) {
         if (s % K == 0)
@@ -802,14 +846,17 @@ extern "C" int llb_adjoint(llb_ctx* c, int nsteps, int every, const void* dev_gf
     }
     void* lam_in = lamA;
     void* lam_out = lamB;
+    // every block adds its dL/domega of each step to its own row; the rows are summed once, at the end
+    size_t used = (size_t)adj_grid(*c).x * c->ny * c->nz;
     for (int k = nseg - 1; k >= 0 && e == cudaSuccess; --k) {
         const int s0 = k * K, s1 = s0 + K < nsteps ? s0 + K : nsteps;
         // recompute the states s0 .. s1-1 of this segment from its checkpoint
-        if (two) {
-            // the two-component step takes any pair of state buffers: step slot to slot
-            e = cudaMemcpyAsync(seg, ck + (size_t)k * sb, sb, cudaMemcpyDeviceToDevice, c->stream);
-            for (int s = s0; s + 1 < s1 && e == cudaSuccess; ++s)
-                e = launch_cg_tiled(*c, seg + (size_t)(s - s0) * sb, seg + (size_t)(s + 1 - s0) * sb);
+        // state s of the segment: the checkpoint itself, then the slots stepped one into the
+        // next (no state is copied), if the step takes any pair of buffers
+        const bool direct = any_buffer(*c);
+        auto state = [&](int s) { return direct && s == s0 ? ck + (size_t)k * sb : seg + (size_t)(s - s0) * sb; };
+        if (direct) {
+            for (int s = s0; s + 1 < s1 && e == cudaSuccess; ++s) e = fwd(*c, state(s), state(s + 1));
         } else {
             e = cudaMemcpyAsync(c->buf[c->cur], ck + (size_t)k * sb, sb, cudaMemcpyDeviceToDevice, c->stream);
             for (int s = s0; s < s1 && e == cudaSuccess; ++s) {
@@ -819,17 +866,16 @@ extern "C" int llb_adjoint(llb_ctx* c, int nsteps, int every, const void* dev_gf
             }
         }
         for (int s = s1 - 1; s >= s0 && e == cudaSuccess; --s) {
-            size_t used = (size_t)adj_grid(*c).x * c->ny * c->nz;
-            e = two ? adj_cg_step(*c, lam_in, seg + (size_t)(s - s0) * sb, lam_out, lamG, rows, &used)
-                    : adj_step(*c, lam_in, seg + (size_t)(s - s0) * sb, lam_out, rows);
-            if (e == cudaSuccess) {
-                k_sum_rows<<<1, 256, 0, c->stream>>>(rows, used, acc);
-                e = cudaGetLastError();
-            }
+            e = two ? adj_cg_step(*c, lam_in, state(s), lam_out, lamG, rows, &used)
+                    : adj_step(*c, lam_in, state(s), lam_out, rows);
             void* tmp = lam_in;
             lam_in = lam_out;
             lam_out = tmp;
         }
+    }
+    if (e == cudaSuccess) {
+        k_sum_rows<<<1, 256, 0, c->stream>>>(rows, used, acc);
+        e = cudaGetLastError();
     }
     // cotangent of the initial state, in canonical form
     if (e == cudaSuccess) {
