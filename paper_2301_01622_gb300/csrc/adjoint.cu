@@ -43,6 +43,7 @@
 #include "lattice.cuh"
 #include "layout.cuh"
 #include "moment_common.cuh"
+#include "twofloat.cuh"
 
 namespace llb {
 namespace {
@@ -52,16 +53,14 @@ constexpr int kAdjThreads = 128;
 // dL/domega term of a node, lam'_A : (j j / rho - A), and its sums.  In FP64 these
 // some 40 operations per node filled the FP64 pipe (two FMA per clock and SM; 79 %
 // busy) and set the time of the adjoint step, 62 of 62 us on 128 x 96 x 64 D3Q19
-// FP32.  For an FP32 state they run on pairs of FP32 numbers, value = h + l with
-// the rounding error of h in l (exact products by FMA, exact sums by Knuth's
-// two-sum), about 2^-46 relative; FP64 states keep FP64.
+// FP32.  For an FP32 state they run on pairs of FP32 numbers (twofloat.cuh); FP64
+// states keep FP64.
 template <class T>
 struct Wide;
 
 template <>
 struct Wide<double> {
     double v = 0.0;
-    __device__ __forceinline__ void add(double h) { v += h; }
     // += a (b r - c)
     __device__ __forceinline__ void add_term(double a, double b, double r, double c) { v += a * (b * r - c); }
     __device__ __forceinline__ double value() const { return v; }
@@ -71,31 +70,15 @@ struct Wide<double> {
 
 template <>
 struct Wide<float> {
-    float h = 0.0f, l = 0.0f;
-    __device__ __forceinline__ void add(float a) {  // two-sum
-        const float s = __fadd_rn(h, a), t = __fsub_rn(s, h);
-        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(a, t)));
-        h = s;
-    }
+    Two v;
     __device__ __forceinline__ void add_term(float a, float b, float r, float c) {
-        const float p = __fmul_rn(b, r), pe = __fmaf_rn(b, r, -p);            // b r = p + pe
-        const float s = __fsub_rn(p, c), t = __fsub_rn(s, p);                 // p - c = s + se
-        const float se = __fsub_rn(__fsub_rn(p, __fsub_rn(s, t)), __fadd_rn(c, t));
-        const float x = __fmul_rn(a, s), xe = __fmaf_rn(a, __fadd_rn(pe, se), __fmaf_rn(a, s, -x));
-        add(x);
-        l = __fadd_rn(l, xe);
+        const Two p = Two::prod(b, r), s = Two::sum(p.h, -c), x = Two::prod(a, s.h);
+        v.add(x.h);
+        v.l = __fadd_rn(v.l, __fmaf_rn(a, __fadd_rn(p.l, s.l), x.l));
     }
-    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-    __device__ __forceinline__ Wide shfl_down(int off) const {
-        Wide o;
-        o.h = __shfl_down_sync(0xffffffffu, h, off);
-        o.l = __shfl_down_sync(0xffffffffu, l, off);
-        return o;
-    }
-    __device__ __forceinline__ void merge(const Wide& o) {
-        add(o.h);
-        l = __fadd_rn(l, o.l);
-    }
+    __device__ __forceinline__ double value() const { return v.value(); }
+    __device__ __forceinline__ Wide shfl_down(int off) const { return {v.shfl_down(off)}; }
+    __device__ __forceinline__ void merge(const Wide& o) { v.add(o.v); }
 };
 
 // Sum of the block's terms, added to its row (fixed order: warp shuffles, then the warps).

@@ -4,7 +4,8 @@
 // canonical (one component): rho, j_x, j_y, j_z, P_xx, P_yy, P_zz, P_xy, P_xz, P_yz
 // shifted storage:           d = rho - 1, j, A = P - cs^2 rho I
 // Equilibrium (second moment of Eq. (5)): P^eq = cs^2 rho I + rho u u, so
-// A^eq = rho u u.  All conversions compute in FP64 and round once.
+// A^eq = rho u u.  All conversions round once: they compute in FP64, or in pairs
+// of floats where both sides are at most FP32.
 // Two components: canonical rho1, rho2, j, P; state rho1, d = rho1 + rho2 - 1,
 // j, A (rho1 needs no shift: it lies in [0, rho]).
 // Canonical buffers are dense; the shifted state follows the context's
@@ -13,11 +14,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "lattice.cuh"
 #include "layout.cuh"
 #include "storage.cuh"
+#include "twofloat.cuh"
 
 namespace llb {
 namespace {
@@ -31,65 +34,150 @@ __device__ __forceinline__ double rdt(const void* p, size_t i, int dt) {
     return dt == LLB_F64 ? rd<double>(p, i) : rd<float>(p, i);
 }
 
-__device__ __forceinline__ void wrt(void* p, size_t i, int dt, double v) {
-    if (dt == LLB_F64) static_cast<double*>(p)[i] = v;
-    else static_cast<float*>(p)[i] = (float)v;
-}
-
 __device__ __forceinline__ bool bad_rho(double r) { return !(r > 0.0) || !isfinite(r); }
 
+// Node i of the dense canonical order (32-bit divisions when the box allows: they
+// are per node and the 64-bit ones cost several times as much).
 __device__ __forceinline__ void decode(const Layout& L, size_t i, int& x, int& y, int& z) {
-    x = (int)(i % L.nx);
-    const size_t r = i / L.nx;
-    y = (int)(r % L.ny);
-    z = (int)(r / L.ny);
-}
-
-template <class T>
-__device__ __forceinline__ void put(T* __restrict__ st, const Layout& L, int x, int y, int z, const double* v) {
-    for_node_and_ghosts(L, x, y, [&](int gx, int gy) {
-        const size_t j = L.at(gx, gy, z);
-#pragma unroll
-        for (int f = 0; f < 10; ++f) st[FieldMap<T, 10>::at(j, f, L.fs)] = to_store<T>(v[f], f);
-    });
-}
-
-// Nodes i0 .. i1-1 of the dense canonical order (whole planes for a z-range).
-template <class T>
-__global__ void k_canon_to_shifted(const void* __restrict__ canon, int cdt, T* __restrict__ st, Layout L,
-                                   int* bad, size_t i0, size_t i1) {
-    const size_t N = (size_t)L.nx * L.ny * L.nz;
-    for (size_t i = i0 + blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
-        double v[10];
-#pragma unroll
-        for (int f = 0; f < 10; ++f) v[f] = rdt(canon, f * N + i, cdt);
-        bool b = bad_rho(v[0]);
-#pragma unroll
-        for (int f = 1; f < 10; ++f) b = b || !isfinite(v[f]);
-        if (b && bad) atomicOr(bad, 1);
-        const double rho = v[0];
-        const double o[10] = {rho - 1.0, v[1], v[2], v[3], v[4] - kCs2 * rho, v[5] - kCs2 * rho,
-                              v[6] - kCs2 * rho, v[7], v[8], v[9]};
-        int x, y, z;
-        decode(L, i, x, y, z);
-        put(st, L, x, y, z, o);
+    if ((i >> 32) == 0) {
+        const unsigned j = (unsigned)i, r = j / (unsigned)L.nx;
+        x = (int)(j - r * (unsigned)L.nx);
+        z = (int)(r / (unsigned)L.ny);
+        y = (int)(r - (unsigned)z * (unsigned)L.ny);
+    } else {
+        x = (int)(i % L.nx);
+        const size_t r = i / L.nx;
+        y = (int)(r % L.ny);
+        z = (int)(r / L.ny);
     }
 }
 
-template <class T>
-__global__ void k_shifted_to_canon(const T* __restrict__ st, void* __restrict__ canon, int cdt, Layout L, size_t i0,
-                                   size_t i1) {
+template <class T, int NF, class V>
+__device__ __forceinline__ void put(T* __restrict__ st, const Layout& L, int x, int y, int z, const V* v) {
+    T t[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+        if constexpr (NF == 10) t[f] = to_store<T>(v[f], f);
+        else t[f] = (T)v[f];
+    for_node_and_ghosts(L, x, y, [&](int gx, int gy) {
+        const size_t j = L.at(gx, gy, z);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) st[FieldMap<T, NF>::at(j, f, L.fs)] = t[f];
+    });
+}
+
+// The maps between canonical and stored values, rounded once.  From FP32 to a
+// state of at most FP32 they run on pairs of floats: in FP64 the two conversions
+// of every value and the arithmetic kept the FP64 pipe 80 % busy and took three
+// times as long as the memory needs.
+template <class C, class T>
+constexpr bool kTwoFloat = std::is_same<C, float>::value && !std::is_same<T, double>::value;
+
+// Total density rho = v[0] (+ v[1]) as rounded value and remainder.
+template <int NC, class V>
+__device__ __forceinline__ void total(const V* v, V& h, V& l) {
+    h = v[0];
+    l = V(0);
+    if constexpr (NC == 2) {
+        if constexpr (std::is_same<V, float>::value) {
+            const Two s = Two::sum(v[0], v[1]);
+            h = s.h;
+            l = s.l;
+        } else {
+            h = v[0] + v[1];
+        }
+    }
+}
+
+__device__ __forceinline__ double less_one(double h, double) { return h - 1.0; }
+__device__ __forceinline__ float less_one(float h, float l) {
+    const Two s = Two::sum(h, -1.0f);
+    return __fadd_rn(s.h, __fadd_rn(s.l, l));
+}
+// P - rho / 3
+__device__ __forceinline__ double less_third(double p, double h, double) { return p - kCs2 * h; }
+__device__ __forceinline__ float less_third(float p, float h, float l) {
+    const Two t = third(h, l), s = Two::sum(p, -t.h);
+    return __fadd_rn(s.h, __fsub_rn(s.l, t.l));
+}
+// A + (1 + d) / 3
+__device__ __forceinline__ double plus_third(double a, double d) { return a + kCs2 * (1.0 + d); }
+__device__ __forceinline__ float plus_third(float a, float d) {
+    const Two r = Two::sum(1.0f, d), t = third(r.h, r.l), s = Two::sum(a, t.h);
+    return __fadd_rn(s.h, __fadd_rn(s.l, t.l));
+}
+__device__ __forceinline__ double one_plus(double d) { return 1.0 + d; }
+__device__ __forceinline__ float one_plus(float d) { return __fadd_rn(1.0f, d); }
+// 1 + d - r1
+__device__ __forceinline__ double other_colour(double d, double r1) { return (1.0 + d) - r1; }
+__device__ __forceinline__ float other_colour(float d, float r1) {
+    const Two r = Two::sum(1.0f, d), s = Two::sum(r.h, -r1);
+    return __fadd_rn(s.h, __fadd_rn(s.l, r.l));
+}
+
+// Nodes i0 .. i1-1 of the dense canonical order (whole planes for a z-range).
+// NC components; canonical rho (rho1, rho2), j, P; state (rho1,) d, j, A.
+template <class C, class T, int NC>
+__global__ void __launch_bounds__(256) k_canon_to_shifted(const C* __restrict__ canon, T* __restrict__ st, Layout L,
+                                                          int* bad, size_t i0, size_t i1) {
+    using V = typename std::conditional<kTwoFloat<C, T>, float, double>::type;
+    constexpr int NF = 9 + NC;
+    const size_t N = (size_t)L.nx * L.ny * L.nz;
+    for (size_t i = i0 + blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
+        V v[NF], o[NF], h, l;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) v[f] = (V)__ldg(canon + f * N + i);
+        total<NC>(v, h, l);
+        // the total density must be positive; a colour density may dip slightly
+        // below zero (the stepped colour-gradient field does so near interfaces)
+        bool b = !(h > V(0)) || (std::is_same<V, double>::value && !isfinite(h));
+#pragma unroll
+        for (int f = 0; f < NF; ++f) b = b || !isfinite(v[f]);
+        if (b && bad) atomicOr(bad, 1);
+        if constexpr (NC == 2) o[0] = v[0];
+        o[NC - 1] = less_one(h, l);
+#pragma unroll
+        for (int f = NC; f < NC + 3; ++f) o[f] = v[f];
+#pragma unroll
+        for (int f = NC + 3; f < NC + 6; ++f) o[f] = less_third(v[f], h, l);
+#pragma unroll
+        for (int f = NC + 6; f < NF; ++f) o[f] = v[f];
+        int x, y, z;
+        decode(L, i, x, y, z);
+        put<T, NF>(st, L, x, y, z, o);
+    }
+}
+
+template <class C, class T, int NC>
+__global__ void __launch_bounds__(256) k_shifted_to_canon(const T* __restrict__ st, C* __restrict__ canon, Layout L,
+                                                          size_t i0, size_t i1) {
+    using V = typename std::conditional<kTwoFloat<C, T>, float, double>::type;
+    constexpr int NF = 9 + NC;
     const size_t N = (size_t)L.nx * L.ny * L.nz;
     for (size_t i = i0 + blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
         int x, y, z;
         decode(L, i, x, y, z);
         const size_t j = L.at(x, y, z);
-        using FM = FieldMap<T, 10>;
-        const double rho = 1.0 + rd_field(st[FM::at(j, 0, L.fs)], 0);
-        wrt(canon, i, cdt, rho);
-        for (int f = 1; f < 4; ++f) wrt(canon, f * N + i, cdt, rd_field(st[FM::at(j, f, L.fs)], f));
-        for (int f = 4; f < 7; ++f) wrt(canon, f * N + i, cdt, rd_field(st[FM::at(j, f, L.fs)], f) + kCs2 * rho);
-        for (int f = 7; f < 10; ++f) wrt(canon, f * N + i, cdt, rd_field(st[FM::at(j, f, L.fs)], f));
+        V v[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const T t = __ldg(st + FieldMap<T, NF>::at(j, f, L.fs));
+            if constexpr (IsNarrow<T>::value) v[f] = cv_field<V>(t, f);
+            else v[f] = (V)t;
+        }
+        const V d = v[NC - 1];
+        if constexpr (NC == 2) {
+            canon[i] = (C)v[0];
+            canon[N + i] = (C)other_colour(d, v[0]);
+        } else {
+            canon[i] = (C)one_plus(d);
+        }
+#pragma unroll
+        for (int f = NC; f < NC + 3; ++f) canon[f * N + i] = (C)v[f];
+#pragma unroll
+        for (int f = NC + 3; f < NC + 6; ++f) canon[f * N + i] = (C)plus_third(v[f], d);
+#pragma unroll
+        for (int f = NC + 6; f < NF; ++f) canon[f * N + i] = (C)v[f];
     }
 }
 
@@ -105,59 +193,7 @@ __global__ void k_equilibrium(const void* __restrict__ rho_p, const void* __rest
                               rho * uz * uz, rho * ux * uy, rho * ux * uz, rho * uy * uz};
         int x, y, z;
         decode(L, i, x, y, z);
-        put(st, L, x, y, z, o);
-    }
-}
-
-// Two components.  canonical: rho1, rho2, j (3), P (6); state: rho1, d = rho1 + rho2 - 1,
-// j (3), A = P - cs^2 rho I (6).
-template <class T>
-__device__ __forceinline__ void put11(T* __restrict__ st, const Layout& L, int x, int y, int z, const double* v) {
-    for_node_and_ghosts(L, x, y, [&](int gx, int gy) {
-        const size_t j = L.at(gx, gy, z);
-#pragma unroll
-        for (int f = 0; f < 11; ++f) st[f * L.fs + j] = (T)v[f];
-    });
-}
-
-template <class T>
-__global__ void k_canon_to_shifted2(const void* __restrict__ canon, int cdt, T* __restrict__ st, Layout L,
-                                    int* bad, size_t i0, size_t i1) {
-    const size_t N = (size_t)L.nx * L.ny * L.nz;
-    for (size_t i = i0 + blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
-        double v[11];
-#pragma unroll
-        for (int f = 0; f < 11; ++f) v[f] = rdt(canon, f * N + i, cdt);
-        const double rho = v[0] + v[1];
-        // the total density must be positive; a colour density may dip slightly
-        // below zero (the stepped colour-gradient field does so near interfaces)
-        bool b = bad_rho(rho) || !isfinite(v[0]) || !isfinite(v[1]);
-#pragma unroll
-        for (int f = 2; f < 11; ++f) b = b || !isfinite(v[f]);
-        if (b && bad) atomicOr(bad, 1);
-        const double o[11] = {v[0], rho - 1.0, v[2], v[3], v[4], v[5] - kCs2 * rho, v[6] - kCs2 * rho,
-                              v[7] - kCs2 * rho, v[8], v[9], v[10]};
-        int x, y, z;
-        decode(L, i, x, y, z);
-        put11(st, L, x, y, z, o);
-    }
-}
-
-template <class T>
-__global__ void k_shifted_to_canon2(const T* __restrict__ st, void* __restrict__ canon, int cdt, Layout L, size_t i0,
-                                    size_t i1) {
-    const size_t N = (size_t)L.nx * L.ny * L.nz;
-    for (size_t i = i0 + blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
-        int x, y, z;
-        decode(L, i, x, y, z);
-        const size_t j = L.at(x, y, z);
-        const double r1 = (double)st[j];
-        const double rho = 1.0 + (double)st[L.fs + j];
-        wrt(canon, i, cdt, r1);
-        wrt(canon, N + i, cdt, rho - r1);
-        for (int f = 2; f < 5; ++f) wrt(canon, f * N + i, cdt, (double)st[f * L.fs + j]);
-        for (int f = 5; f < 8; ++f) wrt(canon, f * N + i, cdt, (double)st[f * L.fs + j] + kCs2 * rho);
-        for (int f = 8; f < 11; ++f) wrt(canon, f * N + i, cdt, (double)st[f * L.fs + j]);
+        put<T, 10>(st, L, x, y, z, o);
     }
 }
 
@@ -175,151 +211,92 @@ __global__ void k_equilibrium2(const void* __restrict__ rho_p, const void* __res
                               rho * uz * uz, rho * ux * uy, rho * ux * uz, rho * uy * uz};
         int x, y, z;
         decode(L, i, x, y, z);
-        put11(st, L, x, y, z, o);
+        put<T, 11>(st, L, x, y, z, o);
     }
 }
 
-int grid_for(const llb_ctx& c) {
-    const size_t want = (c.N + 255) / 256;
+int grid_for(const llb_ctx& c, size_t nodes) {
+    const size_t want = (nodes + 255) / 256;
     const size_t cap = (size_t)(c.num_sms > 0 ? c.num_sms : 148) * 8;
     return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
+// fn(state element type, canonical element type, components)
+template <class T>
+struct Tag {
+    using type = T;
+};
+template <class F>
+void by_types(const llb_ctx& c, int cdt, F&& fn) {
+    auto canon = [&](auto st, auto nc) {
+        if (cdt == LLB_F64) fn(st, Tag<double>{}, nc);
+        else fn(st, Tag<float>{}, nc);
+    };
+    using One = std::integral_constant<int, 1>;
+    using Pair = std::integral_constant<int, 2>;
+    if (c.storage == LLB_F16S) canon(Tag<__half>{}, One{});
+    else if (c.storage == LLB_BF16S) canon(Tag<__nv_bfloat16>{}, One{});
+    else if (c.ncomp == 2 && c.storage == LLB_F64) canon(Tag<double>{}, Pair{});
+    else if (c.ncomp == 2) canon(Tag<float>{}, Pair{});
+    else if (c.storage == LLB_F64) canon(Tag<double>{}, One{});
+    else canon(Tag<float>{}, One{});
+}
+
 }  // namespace
-
-cudaError_t launch_canonical_to_shifted(const llb_ctx& c, const void* canon, int cdt, void* st, int* bad) {
-    if (c.storage == LLB_F16S) {
-        k_canon_to_shifted<__half><<<grid_for(c), 256, 0, c.stream>>>(canon, cdt, static_cast<__half*>(st), c.lay, bad, 0, c.N);
-        return cudaGetLastError();
-    }
-    if (c.storage == LLB_BF16S) {
-        k_canon_to_shifted<__nv_bfloat16><<<grid_for(c), 256, 0, c.stream>>>(canon, cdt, static_cast<__nv_bfloat16*>(st),
-                                                                             c.lay, bad, 0, c.N);
-        return cudaGetLastError();
-    }
-    if (c.ncomp == 2) {
-        if (c.storage == LLB_F64)
-            k_canon_to_shifted2<double><<<grid_for(c), 256, 0, c.stream>>>(canon, cdt, static_cast<double*>(st), c.lay, bad,
-                                                                            0, c.N);
-        else
-            k_canon_to_shifted2<float><<<grid_for(c), 256, 0, c.stream>>>(canon, cdt, static_cast<float*>(st), c.lay, bad,
-                                                                           0, c.N);
-        return cudaGetLastError();
-    }
-    if (c.storage == LLB_F64)
-        k_canon_to_shifted<double><<<grid_for(c), 256, 0, c.stream>>>(canon, cdt, static_cast<double*>(st), c.lay, bad,
-                                                                       0, c.N);
-    else
-        k_canon_to_shifted<float><<<grid_for(c), 256, 0, c.stream>>>(canon, cdt, static_cast<float*>(st), c.lay, bad,
-                                                                      0, c.N);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_shifted_to_canonical(const llb_ctx& c, const void* st, void* canon, int cdt) {
-    if (c.storage == LLB_F16S) {
-        k_shifted_to_canon<__half><<<grid_for(c), 256, 0, c.stream>>>(static_cast<const __half*>(st), canon, cdt, c.lay, 0, c.N);
-        return cudaGetLastError();
-    }
-    if (c.storage == LLB_BF16S) {
-        k_shifted_to_canon<__nv_bfloat16><<<grid_for(c), 256, 0, c.stream>>>(static_cast<const __nv_bfloat16*>(st), canon,
-                                                                             cdt, c.lay, 0, c.N);
-        return cudaGetLastError();
-    }
-    if (c.ncomp == 2) {
-        if (c.storage == LLB_F64)
-            k_shifted_to_canon2<double><<<grid_for(c), 256, 0, c.stream>>>(static_cast<const double*>(st), canon, cdt, c.lay,
-                                                                            0, c.N);
-        else
-            k_shifted_to_canon2<float><<<grid_for(c), 256, 0, c.stream>>>(static_cast<const float*>(st), canon, cdt, c.lay,
-                                                                           0, c.N);
-        return cudaGetLastError();
-    }
-    if (c.storage == LLB_F64)
-        k_shifted_to_canon<double><<<grid_for(c), 256, 0, c.stream>>>(static_cast<const double*>(st), canon, cdt, c.lay,
-                                                                       0, c.N);
-    else
-        k_shifted_to_canon<float><<<grid_for(c), 256, 0, c.stream>>>(static_cast<const float*>(st), canon, cdt, c.lay,
-                                                                      0, c.N);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_canonical_to_shifted_range(const llb_ctx& c, const void* canon, int cdt, void* st, int* bad, int zlo,
                                               int zhi, cudaStream_t s) {
     const size_t per = (size_t)c.nx * c.ny, i0 = per * zlo, i1 = per * zhi;
-    const int grid = (int)std::min<size_t>((i1 - i0 + 255) / 256, (size_t)c.num_sms * 8);
-    if (c.ncomp == 2) {
-        if (c.storage == LLB_F64)
-            k_canon_to_shifted2<double><<<grid, 256, 0, s>>>(canon, cdt, static_cast<double*>(st), c.lay, bad, i0, i1);
-        else
-            k_canon_to_shifted2<float><<<grid, 256, 0, s>>>(canon, cdt, static_cast<float*>(st), c.lay, bad, i0, i1);
-        return cudaGetLastError();
-    }
-    switch (c.storage) {
-        case LLB_F64:
-            k_canon_to_shifted<double><<<grid, 256, 0, s>>>(canon, cdt, static_cast<double*>(st), c.lay, bad, i0, i1);
-            break;
-        case LLB_F16S:
-            k_canon_to_shifted<__half><<<grid, 256, 0, s>>>(canon, cdt, static_cast<__half*>(st), c.lay, bad, i0, i1);
-            break;
-        case LLB_BF16S:
-            k_canon_to_shifted<__nv_bfloat16><<<grid, 256, 0, s>>>(canon, cdt, static_cast<__nv_bfloat16*>(st), c.lay,
-                                                                  bad, i0, i1);
-            break;
-        default:
-            k_canon_to_shifted<float><<<grid, 256, 0, s>>>(canon, cdt, static_cast<float*>(st), c.lay, bad, i0, i1);
-    }
+    by_types(c, cdt, [&](auto t, auto u, auto nc) {
+        using T = typename decltype(t)::type;
+        using C = typename decltype(u)::type;
+        k_canon_to_shifted<C, T, decltype(nc)::value><<<grid_for(c, i1 - i0), 256, 0, s>>>(
+            static_cast<const C*>(canon), static_cast<T*>(st), c.lay, bad, i0, i1);
+    });
     return cudaGetLastError();
 }
 
 cudaError_t launch_shifted_to_canonical_range(const llb_ctx& c, const void* st, void* canon, int cdt, int zlo, int zhi,
                                               cudaStream_t s) {
     const size_t per = (size_t)c.nx * c.ny, i0 = per * zlo, i1 = per * zhi;
-    const int grid = (int)std::min<size_t>((i1 - i0 + 255) / 256, (size_t)c.num_sms * 8);
-    if (c.ncomp == 2) {
-        if (c.storage == LLB_F64)
-            k_shifted_to_canon2<double><<<grid, 256, 0, s>>>(static_cast<const double*>(st), canon, cdt, c.lay, i0, i1);
-        else
-            k_shifted_to_canon2<float><<<grid, 256, 0, s>>>(static_cast<const float*>(st), canon, cdt, c.lay, i0, i1);
-        return cudaGetLastError();
-    }
-    switch (c.storage) {
-        case LLB_F64:
-            k_shifted_to_canon<double><<<grid, 256, 0, s>>>(static_cast<const double*>(st), canon, cdt, c.lay, i0, i1);
-            break;
-        case LLB_F16S:
-            k_shifted_to_canon<__half><<<grid, 256, 0, s>>>(static_cast<const __half*>(st), canon, cdt, c.lay, i0, i1);
-            break;
-        case LLB_BF16S:
-            k_shifted_to_canon<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(st), canon, cdt,
-                                                                  c.lay, i0, i1);
-            break;
-        default:
-            k_shifted_to_canon<float><<<grid, 256, 0, s>>>(static_cast<const float*>(st), canon, cdt, c.lay, i0, i1);
-    }
+    by_types(c, cdt, [&](auto t, auto u, auto nc) {
+        using T = typename decltype(t)::type;
+        using C = typename decltype(u)::type;
+        k_shifted_to_canon<C, T, decltype(nc)::value><<<grid_for(c, i1 - i0), 256, 0, s>>>(
+            static_cast<const T*>(st), static_cast<C*>(canon), c.lay, i0, i1);
+    });
     return cudaGetLastError();
+}
+
+cudaError_t launch_canonical_to_shifted(const llb_ctx& c, const void* canon, int cdt, void* st, int* bad) {
+    return launch_canonical_to_shifted_range(c, canon, cdt, st, bad, 0, c.nz, c.stream);
+}
+
+cudaError_t launch_shifted_to_canonical(const llb_ctx& c, const void* st, void* canon, int cdt) {
+    return launch_shifted_to_canonical_range(c, st, canon, cdt, 0, c.nz, c.stream);
 }
 
 cudaError_t launch_equilibrium(const llb_ctx& c, const void* rho, const void* u, int dt, void* st, int* bad) {
     if (c.storage == LLB_F16S) {
-        k_equilibrium<__half><<<grid_for(c), 256, 0, c.stream>>>(rho, u, dt, static_cast<__half*>(st), c.lay, bad);
+        k_equilibrium<__half><<<grid_for(c, c.N), 256, 0, c.stream>>>(rho, u, dt, static_cast<__half*>(st), c.lay, bad);
         return cudaGetLastError();
     }
     if (c.storage == LLB_BF16S) {
-        k_equilibrium<__nv_bfloat16><<<grid_for(c), 256, 0, c.stream>>>(rho, u, dt, static_cast<__nv_bfloat16*>(st),
+        k_equilibrium<__nv_bfloat16><<<grid_for(c, c.N), 256, 0, c.stream>>>(rho, u, dt, static_cast<__nv_bfloat16*>(st),
                                                                         c.lay, bad);
         return cudaGetLastError();
     }
     if (c.ncomp == 2) {
         if (c.storage == LLB_F64)
-            k_equilibrium2<double><<<grid_for(c), 256, 0, c.stream>>>(rho, u, dt, static_cast<double*>(st), c.lay, bad);
+            k_equilibrium2<double><<<grid_for(c, c.N), 256, 0, c.stream>>>(rho, u, dt, static_cast<double*>(st), c.lay, bad);
         else
-            k_equilibrium2<float><<<grid_for(c), 256, 0, c.stream>>>(rho, u, dt, static_cast<float*>(st), c.lay, bad);
+            k_equilibrium2<float><<<grid_for(c, c.N), 256, 0, c.stream>>>(rho, u, dt, static_cast<float*>(st), c.lay, bad);
         return cudaGetLastError();
     }
     if (c.storage == LLB_F64)
-        k_equilibrium<double><<<grid_for(c), 256, 0, c.stream>>>(rho, u, dt, static_cast<double*>(st), c.lay, bad);
+        k_equilibrium<double><<<grid_for(c, c.N), 256, 0, c.stream>>>(rho, u, dt, static_cast<double*>(st), c.lay, bad);
     else
-        k_equilibrium<float><<<grid_for(c), 256, 0, c.stream>>>(rho, u, dt, static_cast<float*>(st), c.lay, bad);
+        k_equilibrium<float><<<grid_for(c, c.N), 256, 0, c.stream>>>(rho, u, dt, static_cast<float*>(st), c.lay, bad);
     return cudaGetLastError();
 }
 

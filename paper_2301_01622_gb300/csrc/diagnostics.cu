@@ -6,16 +6,19 @@
 // reduces in registers, then warp shuffles, then across the block's warps
 // through shared memory, and writes one row of partials per block to a
 // scratch array.  Pass 2: one block reduces the rows in a fixed order.  The
-// result is deterministic for a given grid.
+// result is deterministic for a given grid.  The sums are FP64 for FP64 states
+// and carry at least its 46 leading bits for the others.
 #include <cuda_runtime.h>
 
 #include <cfloat>
 #include <mutex>
+#include <type_traits>
 
 #include "internal.h"
 #include "lattice.cuh"
 #include "layout.cuh"
 #include "storage.cuh"
+#include "twofloat.cuh"
 
 namespace llb {
 namespace {
@@ -26,12 +29,6 @@ constexpr int kRow = 9;  // sum d, sum jx, sum jy, sum jz, sum rho_in, n_in, min
 struct Part {
     double v[kRow];
 };
-
-__device__ __forceinline__ void part_init(Part& p) {
-#pragma unroll
-    for (int k = 0; k < kRow; ++k) p.v[k] = 0.0;
-    p.v[6] = DBL_MAX;
-}
 
 __device__ __forceinline__ void part_merge(Part& a, const Part& b) {
 #pragma unroll
@@ -52,75 +49,199 @@ __device__ __forceinline__ Part warp_reduce(Part p) {
     return p;
 }
 
-// Block-wide reduction; the result is valid in thread 0.
-__device__ Part block_reduce(Part p) {
-    __shared__ double sh[kDiagThreads / 32][kRow];
-    p = warp_reduce(p);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int k = 0; k < kRow; ++k) sh[wid][k] = p.v[k];
-    __syncthreads();
-    if (wid == 0) {
-        Part q;
-        part_init(q);
-        if (lane < kDiagThreads / 32)
-            for (int k = 0; k < kRow; ++k) q.v[k] = sh[lane][k];
-        p = warp_reduce(q);
-    }
-    return p;
-}
+// Sums of one thread.  States and inputs of at most FP32 are summed as pairs of
+// floats (twofloat.cuh): the FP64 form kept the FP64 pipe 79 % busy and took 106 us
+// for the 92 MB of a 128^3 two-component state.
+template <bool WIDE>
+struct Sums;
 
-// Row of partial sums: (sum d, sum j, sum of the droplet density over nodes
-// where it exceeds 0.5, their count, min rho, non-finite flag, sum rho1).
+template <>
+struct Sums<true> {  // FP64 values
+    double v[kRow];
+    __device__ __forceinline__ Sums() {
+        for (int k = 0; k < kRow; ++k) v[k] = 0.0;
+        v[6] = DBL_MAX;
+    }
+    __device__ __forceinline__ void node(double d, double jx, double jy, double jz, double drop, bool two, bool finite) {
+        const double rho = 1.0 + d;
+        v[0] += d;
+        v[1] += jx;
+        v[2] += jy;
+        v[3] += jz;
+        if (drop > 0.5) {
+            v[4] += drop;
+            v[5] += 1.0;
+        }
+        v[6] = fmin(v[6], rho);
+        if (!finite) v[7] = 1.0;
+        if (two) v[8] += drop;
+    }
+    // one component from canonical rho (the sums are of the density as given)
+    __device__ __forceinline__ void canonical(double rho, double jx, double jy, double jz, bool finite) {
+        v[0] += rho - 1.0;
+        v[1] += jx;
+        v[2] += jy;
+        v[3] += jz;
+        if (rho > 0.5) {
+            v[4] += rho;
+            v[5] += 1.0;
+        }
+        v[6] = fmin(v[6], rho);
+        if (!finite) v[7] = 1.0;
+    }
+    __device__ __forceinline__ Part row() const {
+        Part p;
+        for (int k = 0; k < kRow; ++k) p.v[k] = v[k];
+        return warp_reduce(p);
+    }
+};
+
+template <>
+struct Sums<false> {  // FP32 values
+    Two d, jx, jy, jz, in, all;  // in: sum of the droplet density (one component: of d) where it exceeds 0.5
+    float dmin = FLT_MAX, rmin = FLT_MAX;
+    unsigned n_in = 0, bad = 0;
+    bool two = false;
+    __device__ __forceinline__ void node(float dv, float x, float y, float z, float drop, bool two_, bool finite) {
+        two = two_;
+        d.add(dv);
+        jx.add(x);
+        jy.add(y);
+        jz.add(z);
+        // one component: rho = 1 + d > 0.5; its 1 is added with the count
+        const float v = two_ ? drop : dv;
+        if (v > (two_ ? 0.5f : -0.5f)) {
+            in.add(v);
+            ++n_in;
+        }
+        dmin = fminf(dmin, dv);
+        if (!finite) bad = 1;
+        if (two_) all.add(drop);
+    }
+    __device__ __forceinline__ void canonical(float rho, float x, float y, float z, bool finite) {
+        const Two dv = Two::sum(rho, -1.0f);
+        d.add(dv);
+        jx.add(x);
+        jy.add(y);
+        jz.add(z);
+        if (rho > 0.5f) {
+            in.add(dv);
+            ++n_in;
+        }
+        rmin = fminf(rmin, rho);
+        if (!finite) bad = 1;
+    }
+    // Sums of the warp, in lane 0.
+    __device__ __forceinline__ Part row() {
+        double n = 0.0;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            d.add(d.shfl_down(off));
+            jx.add(jx.shfl_down(off));
+            jy.add(jy.shfl_down(off));
+            jz.add(jz.shfl_down(off));
+            in.add(in.shfl_down(off));
+            if (two) all.add(all.shfl_down(off));
+            dmin = fminf(dmin, __shfl_down_sync(0xffffffffu, dmin, off));
+            rmin = fminf(rmin, __shfl_down_sync(0xffffffffu, rmin, off));
+            bad |= __shfl_down_sync(0xffffffffu, bad, off);
+        }
+        n = (double)__reduce_add_sync(0xffffffffu, n_in);
+        Part p;
+        p.v[0] = d.value();
+        p.v[1] = jx.value();
+        p.v[2] = jy.value();
+        p.v[3] = jz.value();
+        p.v[4] = in.value() + (two ? 0.0 : n);
+        p.v[5] = n;
+        p.v[6] = fmin(dmin == FLT_MAX ? DBL_MAX : 1.0 + (double)dmin, rmin == FLT_MAX ? DBL_MAX : (double)rmin);
+        p.v[7] = (double)bad;
+        p.v[8] = all.value();
+        return p;
+    }
+};
+
+// Row of partial sums of the block: (sum d, sum j, sum of the droplet density over
+// nodes where it exceeds 0.5, their count, min rho, non-finite flag, sum rho1).
 // The droplet density is rho for one component and rho1 for two (state
 // rho1, d, j, A; rho2 = 1 + d - rho1 is recovered from the sums).
+template <bool WIDE>
+__device__ __forceinline__ void write_row(Sums<WIDE>& s, bool two, double* __restrict__ row) {
+    __shared__ double sh[kDiagThreads / 32][kRow];
+    if constexpr (!WIDE) s.two = two;  // a thread without nodes takes part in the same shuffles
+    const Part p = s.row();
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < kRow; ++k) sh[threadIdx.x >> 5][k] = p.v[k];
+    __syncthreads();
+    if (threadIdx.x < kRow) {
+        const int k = threadIdx.x;
+        double v = sh[0][k];
+        for (int w = 1; w < kDiagThreads / 32; ++w) v = k == 6 ? fmin(v, sh[w][k]) : k == 7 ? fmax(v, sh[w][k]) : v + sh[w][k];
+        row[k] = v;
+    }
+}
+
 template <class T, int NC>
 __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(const T* __restrict__ m, Layout L,
                                                                double* __restrict__ rows) {
-    Part p;
-    part_init(p);
+    constexpr bool WIDE = std::is_same<T, double>::value;
+    using V = typename std::conditional<WIDE, double, float>::type;
+    using FM = FieldMap<T, 9 + NC>;
+    Sums<WIDE> s;
     const size_t N = (size_t)L.nx * L.ny * L.nz, F = L.fs;
-    constexpr int o = NC == 2 ? 1 : 0;  // field offset of d
     for (size_t n = blockIdx.x * (size_t)kDiagThreads + threadIdx.x; n < N; n += (size_t)gridDim.x * kDiagThreads) {
-        const int x = (int)(n % L.nx);
-        const size_t r = n / L.nx;
-        const size_t i = L.at(x, (int)(r % L.ny), (int)(r / L.ny));
-        using FM = FieldMap<T, NC == 2 ? 11 : 10>;
-        const double d = rd_field(m[FM::at(i, o, F)], 0);
-        const double jx = rd_field(m[FM::at(i, o + 1, F)], 1), jy = rd_field(m[FM::at(i, o + 2, F)], 2),
-                     jz = rd_field(m[FM::at(i, o + 3, F)], 3);
-        const double rho = 1.0 + d;
-        const double drop = NC == 2 ? rd_field(m[FM::at(i, 0, F)], 0) : rho;
-        p.v[0] += d;
-        p.v[1] += jx;
-        p.v[2] += jy;
-        p.v[3] += jz;
-        if (drop > 0.5) {
-            p.v[4] += drop;
-            p.v[5] += 1.0;
+        size_t r;
+        int x, y, z;
+        if ((N >> 32) == 0) {  // 32-bit divisions when the box allows
+            const unsigned q = (unsigned)n / (unsigned)L.nx;
+            x = (int)((unsigned)n - q * (unsigned)L.nx);
+            z = (int)(q / (unsigned)L.ny);
+            y = (int)(q - (unsigned)z * (unsigned)L.ny);
+        } else {
+            x = (int)(n % L.nx);
+            r = n / L.nx;
+            y = (int)(r % L.ny);
+            z = (int)(r / L.ny);
         }
-        p.v[6] = fmin(p.v[6], rho);
-        if (NC == 2) p.v[8] += drop;
-        bool finite = isfinite(d) && isfinite(jx) && isfinite(jy) && isfinite(jz) && isfinite(drop);
+        const size_t i = L.at(x, y, z);
+        V v[9 + NC];
+        bool finite = true;
 #pragma unroll
-        for (int f = o + 4; f < o + 10; ++f) finite = finite && isfinite(rd_field(m[FM::at(i, f, F)], f - o));
-        if (!finite) p.v[7] = 1.0;
+        for (int f = 0; f < 9 + NC; ++f) {
+            const T t = __ldg(m + FM::at(i, f, F));
+            if constexpr (IsNarrow<T>::value) v[f] = cv_field<V>(t, f);
+            else v[f] = (V)t;
+            finite = finite && isfinite(v[f]);
+        }
+        s.node(v[NC - 1], v[NC], v[NC + 1], v[NC + 2], NC == 2 ? v[0] : V(1) + v[0], NC == 2, finite);
     }
-    p = block_reduce(p);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < kRow; ++k) rows[(size_t)blockIdx.x * kRow + k] = p.v[k];
+    write_row(s, NC == 2, rows + (size_t)blockIdx.x * kRow);
 }
 
-__global__ void __launch_bounds__(kDiagThreads) k_diag_final(const double* __restrict__ rows, int nrows, size_t N,
+// Sum of the rows, in a fixed order.
+__global__ void __launch_bounds__(32 * kRow) k_diag_final(const double* __restrict__ rows, int nrows, size_t N,
                                                              int ncomp, llb_diag* __restrict__ out) {
-    Part p;
-    part_init(p);
-    for (int r = threadIdx.x; r < nrows; r += kDiagThreads) {
-        Part q;
-        for (int k = 0; k < kRow; ++k) q.v[k] = rows[(size_t)r * kRow + k];
-        part_merge(p, q);
+    // 32 threads per column read the rows in order (coalesced), then a warp per column joins them
+    __shared__ double part[kRow][33], sh[kRow];
+    auto join = [](int k, double a, double b) { return k == 6 ? fmin(a, b) : k == 7 ? fmax(a, b) : a + b; };
+    {
+        const int k = threadIdx.x % kRow;
+        double v = k == 6 ? DBL_MAX : 0.0;
+#pragma unroll 8
+        for (int i = threadIdx.x; i < nrows * kRow; i += 32 * kRow) v = join(k, v, rows[i]);
+        part[k][threadIdx.x / kRow] = v;
     }
-    p = block_reduce(p);
+    __syncthreads();
+    {
+        const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        double v = part[k][lane];
+        for (int off = 16; off > 0; off >>= 1) v = join(k, v, __shfl_down_sync(0xffffffffu, v, off));
+        if (lane == 0) sh[k] = v;
+    }
+    __syncthreads();
+    Part p;
+    if (threadIdx.x == 0)
+        for (int q = 0; q < kRow; ++q) p.v[q] = sh[q];
     if (threadIdx.x == 0) {
         if (ncomp == 2) {
             out->mass[0] = p.v[8];
@@ -171,7 +292,7 @@ cudaError_t launch_diagnostics(const llb_ctx& c, const void* mom, void* scratch,
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_diag_final<<<1, kDiagThreads, 0, c.stream>>>(rows, nb, c.N, c.ncomp, dev_out);
+    k_diag_final<<<1, 32 * kRow, 0, c.stream>>>(rows, nb, c.N, c.ncomp, dev_out);
     return cudaGetLastError();
 }
 
@@ -211,31 +332,21 @@ static __device__ __align__(256) StaticScratch g_diag_scratch;
 template <class T>
 __global__ void __launch_bounds__(kDiagThreads) k_diag_partial_canonical(const T* __restrict__ m, size_t N,
                                                                          double* __restrict__ rows) {
-    Part p;
-    part_init(p);
+    constexpr bool WIDE = std::is_same<T, double>::value;
+    Sums<WIDE> s;
     const size_t lo = (size_t)blockIdx.x * kStaticNodesPerRow;
     const size_t hi = lo + kStaticNodesPerRow < N ? lo + kStaticNodesPerRow : N;
     for (size_t i = lo + threadIdx.x; i < hi; i += kDiagThreads) {
-        const double rho = (double)m[i];
-        const double d = rho - 1.0;
-        const double jx = (double)m[N + i], jy = (double)m[2 * N + i], jz = (double)m[3 * N + i];
-        p.v[0] += d;
-        p.v[1] += jx;
-        p.v[2] += jy;
-        p.v[3] += jz;
-        if (rho > 0.5) {
-            p.v[4] += rho;
-            p.v[5] += 1.0;
-        }
-        p.v[6] = fmin(p.v[6], rho);
-        bool finite = isfinite(rho) && isfinite(jx) && isfinite(jy) && isfinite(jz);
+        T v[10];
+        bool finite = true;
 #pragma unroll
-        for (int f = 4; f < 10; ++f) finite = finite && isfinite((double)m[f * N + i]);
-        if (!finite) p.v[7] = 1.0;
+        for (int f = 0; f < 10; ++f) {
+            v[f] = __ldg(m + f * N + i);
+            finite = finite && isfinite(v[f]);
+        }
+        s.canonical(v[0], v[1], v[2], v[3], finite);
     }
-    p = block_reduce(p);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < kRow; ++k) rows[(size_t)blockIdx.x * kRow + k] = p.v[k];
+    write_row(s, false, rows + (size_t)blockIdx.x * kRow);
 }
 
 constexpr int kMaxDevices = 64;
@@ -281,7 +392,7 @@ extern "C" int llb_diagnostics_noalloc(const void* dev_m, int dtype, int nx, int
         k_diag_partial_canonical<float><<<nb, kDiagThreads, 0, s>>>(static_cast<const float*>(dev_m), N,
                                                                      scratch->rows);
     if (cudaGetLastError() != cudaSuccess) return LLB_ECUDA;
-    k_diag_final<<<1, kDiagThreads, 0, s>>>(scratch->rows, nb, N, 1, &scratch->out);
+    k_diag_final<<<1, 32 * kRow, 0, s>>>(scratch->rows, nb, N, 1, &scratch->out);
     if (cudaGetLastError() != cudaSuccess) return LLB_ECUDA;
     if (cudaMemcpyAsync(host_out, &scratch->out, sizeof(llb_diag), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
