@@ -99,9 +99,10 @@ typedef struct llb_params {
     int scheme;       /* LLB_SCHEME_* (default LLB_SCHEME_MOMENT)            */
     int kernel;       /* LLB_KERNEL_* (default LLB_KERNEL_AUTO)              */
     int variant;      /* tuning variant, 0 = default.  One component, FP32:
-                         tiled kernel 0..5 (TMA L2 prefetch, IEEE 1/rho,
-                         64x8 and 32x8 tiles, split-phase plane barrier),
-                         TMA kernel 0..2 (ring depth, tile); the other
+                         tiled kernel 0..5 (0: two nodes per thread, tile
+                         30x6; one node per thread, 64x4: TMA L2 prefetch,
+                         IEEE 1/rho, then 64x8 and 32x8 tiles, 64x4 with a
+                         split-phase plane barrier), TMA kernel 0..2 (ring depth, tile); the other
                          storage types have one shape per kernel.  Two
                          components, FP32: 0..5 (0: two nodes per thread,
                          tile 28x10, approximate FP32 quotients; one node per

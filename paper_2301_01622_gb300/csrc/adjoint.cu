@@ -738,7 +738,7 @@ int grid_n(const llb_ctx& c) {
 cudaError_t fwd(const llb_ctx& c, const void* in, void* out) {
     return c.ncomp == 2                   ? launch_cg_tiled(c, in, out)
            : c.kernel == LLB_KERNEL_TMA   ? launch_moment_tma(c, c.cur, out)
-           : c.kernel == LLB_KERNEL_TILED ? launch_moment_tiled(c, c.cur, in, out)
+           : c.kernel == LLB_KERNEL_TILED ? launch_moment_tiled(c, c.cur, in, out, false)
                                           : launch_moment_direct(c, in, out);
 }
 

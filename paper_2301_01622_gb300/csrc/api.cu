@@ -193,14 +193,15 @@ int check_bad_flag(llb_ctx* c) {
     return LLB_OK;
 }
 
-// Launch one step from buffer `cur` into the other copy, without flipping.
-cudaError_t launch_one(llb_ctx* c, int cur) {
+// Launch one step from buffer `cur` into the other copy, without flipping.  last: the
+// step whose result stays the current state when the call returns.
+cudaError_t launch_one(llb_ctx* c, int cur, bool last) {
     const void* in = c->buf[cur];
     void* out = c->buf[1 - cur];
     if (c->ncomp == 2 && c->scheme == LLB_SCHEME_MOMENT) return launch_cg_tiled(*c, in, out);
     if (c->scheme == LLB_SCHEME_MOMENT)
         return c->kernel == LLB_KERNEL_TMA     ? launch_moment_tma(*c, cur, out)
-               : c->kernel == LLB_KERNEL_TILED ? launch_moment_tiled(*c, cur, in, out)
+               : c->kernel == LLB_KERNEL_TILED ? launch_moment_tiled(*c, cur, in, out, last)
                                                : launch_moment_direct(*c, in, out);
     return launch_population_step(*c, in, out, c->scheme == LLB_SCHEME_POPULATION_BGK);
 }
@@ -424,7 +425,7 @@ int llb_step(llb_ctx* c, int nsteps) {
     if (c->in_batch) return fail(c, LLB_EINVAL, "this box belongs to a batch: step it with llb_batch_step");
     if (nsteps < 0) return fail(c, LLB_EINVAL, "nsteps must be >= 0");
     for (int s = 0; s < nsteps; ++s) {
-        const cudaError_t e = launch_one(c, c->cur);
+        const cudaError_t e = launch_one(c, c->cur, s == nsteps - 1);
         if (e != cudaSuccess) return cuda_fail(c, e, "step kernel");
         c->cur = 1 - c->cur;
         ++c->t;
@@ -451,7 +452,7 @@ int llb_step_graph(llb_ctx* c, int nsteps) {
         cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         int cur = k;
         for (int s = 0; s < nsteps && e == cudaSuccess; ++s) {
-            e = launch_one(c, cur);
+            e = launch_one(c, cur, s == nsteps - 1);
             cur = 1 - cur;
         }
         cudaGraph_t g = nullptr;
@@ -501,9 +502,9 @@ int llb_autotune(llb_ctx* c, int trials, int* kernel, int* variant) {
     for (int i = 0; i < nc; ++i) {
         if (!configure(c, cands[i].kernel, cands[i].variant)) continue;
         // every trial recomputes step t -> t+1 into the spare copy: the state does not move
-        cudaError_t e = launch_one(c, c->cur);
+        cudaError_t e = launch_one(c, c->cur, true);
         if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-        for (int r = 0; r < trials && e == cudaSuccess; ++r) e = launch_one(c, c->cur);
+        for (int r = 0; r < trials && e == cudaSuccess; ++r) e = launch_one(c, c->cur, true);
         if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.0f;

@@ -22,13 +22,6 @@
 // whole tile's.)  The rows above and below are doubled in the exchange (one copy for
 // every other plane), so that the halo warp publishes plane s + 1 while the tile
 // warps still pull plane s.
-//
-// Exchange.  Along an in-plane direction (cx, cy) the populations with c_z = -1,
-// 0, 1 are c0 + zz - c1, c0, c0 + zz + c1 with
-//   c0 = s + [cx] a_xx + [cy] a_yy + cx j_x + cy j_y + cx cy a_xy,
-//   c1 = j_z + cx a_xz + cy a_yz, zz = a_zz (scaled moments of pair_march.cuh),
-// so a node publishes c0 and c1 per direction and zz once, and the pull sums c0,
-// c0 + zz and c1 separately before it forms the three planes.
 #pragma once
 
 #include <algorithm>
@@ -43,7 +36,7 @@ namespace cg {
 // Constants of the scaled collision: w = the smallest weight.
 struct PairK {
     float ka, kc, ko;          // 4.5 w (1 - omega), 9 w (1 - omega), 4.5 w omega
-    float w, wj;               // w, 3 w
+    float w, wj, wj2;          // w, 3 w and what rounding it left
     float kg, bw, kf;          // 0.5 w A_s, beta w, 9 w (1 - omega / 2)
     float A_h, g_min, g_nci, eps2;
     int h_c;
@@ -58,6 +51,7 @@ PairK pair_constants(const llb_ctx& c) {
     k.ko = (float)(4.5 * w * om);
     k.w = (float)w;
     k.wj = (float)(3.0 * w);
+    k.wj2 = (float)(3.0 * w - (double)k.wj);
     k.kg = (float)(0.5 * w * c.params.A_s);
     k.bw = (float)(c.params.beta * w);
     k.kf = (float)(9.0 * w * (1.0 - 0.5 * om));
@@ -172,16 +166,16 @@ __device__ __forceinline__ Src collide_pair(float2 r1, float2 d, const float2* m
         s.c.xy = fma(ux, fy, fma(uy, fx, s.c.xy));
         s.c.xz = fma(ux, fz, fma(uz, fx, s.c.xz));
         s.c.yz = fma(uy, fz, fma(uz, fy, s.c.yz));
-        s.c.jx = mul(k.wj, add(jx, fx));
-        s.c.jy = mul(k.wj, add(jy, fy));
-        s.c.jz = mul(k.wj, add(jz, fz));
+        s.c.jx = col_j(k.wj, k.wj2, add(jx, fx));
+        s.c.jy = col_j(k.wj, k.wj2, add(jy, fy));
+        s.c.jz = col_j(k.wj, k.wj2, add(jz, fz));
     } else {
         collide(jx, jy, jz);
-        s.c.jx = mul(k.wj, jx);
-        s.c.jy = mul(k.wj, jy);
-        s.c.jz = mul(k.wj, jz);
+        s.c.jx = col_j(k.wj, k.wj2, jx);
+        s.c.jy = col_j(k.wj, k.wj2, jy);
+        s.c.jz = col_j(k.wj, k.wj2, jz);
     }
-    s.c.s = fma(-(1.0f / 3.0f), add(add(s.c.xx, s.c.yy), s.c.zz), mul(k.w, d));
+    s.c.s = col_s(s.c.xx, s.c.yy, s.c.zz, mul(k.w, d));
     // e = beta rho1 rho2 / rho
     const float2 rho2 = add(sub(make_float2(1.0f, 1.0f), r1), d);
     const float2 e = mul(mul(mul(k.bw, s.r1), rho2), ig);
@@ -200,10 +194,6 @@ struct CgTile {
     static constexpr int PN = W * (H + 4);               // phi: pair rows -2 .. H+1
     static constexpr bool kC = pk::Shells<L>::corners;
     static constexpr int N4 = kC ? 8 : 4, N2 = kC ? 0 : 4;  // directions with (c0, c1), with c0 only
-    // in-plane directions: (1,0) (-1,0) (0,1) (0,-1) (1,1) (-1,-1) (1,-1) (-1,1)
-    static constexpr int dir(int cx, int cy) {
-        return cy == 0 ? (cx > 0 ? 0 : 1) : cx == 0 ? (cy > 0 ? 2 : 3) : cx == cy ? (cx > 0 ? 4 : 5) : cx > 0 ? 6 : 7;
-    }
     // staged boxes: columns x0-4 .. x0+31; (rho1, d) rows -2 .. BY+1, four planes;
     // the other nine fields rows -1 .. BY, two planes; results: columns x0 .. x0+27
     static constexpr int SX = 36, RR = BY + 4, RM = BY + 2;
@@ -218,55 +208,6 @@ struct CgTile {
     static constexpr int smem_bytes = BAR_OFF + 16 + 128;  // two mbarriers; slack to align the base to 128 bytes
     static_assert(BX % 4 == 0, "box starts on 16-byte boundaries");
 };
-
-// Call put(Dir, c0, c1) for every in-plane direction with want(cx, cy).
-template <class Want, class Put>
-__device__ __forceinline__ void emit_plane(const pk::Col<float2>& c, Want want, Put put) {
-    using namespace pk;
-    const float2 ex = add(c.s, c.xx), ey = add(c.s, c.yy), exy = add(ex, c.yy);
-    const float2 zp = add(c.jz, c.xz), zm = sub(c.jz, c.xz);
-    const float2 u = add(exy, c.xy), v = sub(exy, c.xy), p = add(c.jx, c.jy), m = sub(c.jx, c.jy);
-    auto one = [&](auto d, float2 c0, float2 c1) {
-        using D = decltype(d);
-        if (want(D::cx, D::cy)) put(d, c0, c1);
-    };
-    one(Dir<1, 0, 0>{}, add(ex, c.jx), zp);
-    one(Dir<-1, 0, 0>{}, sub(ex, c.jx), zm);
-    one(Dir<0, 1, 0>{}, add(ey, c.jy), add(c.jz, c.yz));
-    one(Dir<0, -1, 0>{}, sub(ey, c.jy), sub(c.jz, c.yz));
-    one(Dir<1, 1, 0>{}, add(u, p), add(zp, c.yz));
-    one(Dir<-1, -1, 0>{}, sub(u, p), sub(zm, c.yz));
-    one(Dir<1, -1, 0>{}, add(v, m), sub(zp, c.yz));
-    one(Dir<-1, 1, 0>{}, sub(v, m), add(zm, c.yz));
-}
-
-// Sums over the eight neighbours of one published quantity, in the moments a
-// plane accumulates (shell factors own : axis : diag; no diagonals if !D).
-template <bool D>
-__device__ __forceinline__ pk::PlaneSum<float2> plane_sum(float own, float axis, float diag, float2 o, float2 ax,
-                                                          float2 bx, float2 ay, float2 by, float2 pp, float2 mm,
-                                                          float2 pm, float2 mp) {
-    using namespace pk;
-    PlaneSum<float2> r;
-    const float2 sx = add(ax, bx), dx = sub(ax, bx), sy = add(ay, by), dy = sub(ay, by);
-    if constexpr (D) {
-        const float2 a = add(pp, mm), b = add(pm, mp), c = sub(pp, mm), e = sub(pm, mp);
-        const float2 sd = add(a, b);
-        r.xx = fma(axis, sx, sd);
-        r.yy = fma(axis, sy, sd);
-        r.jx = fma(axis, dx, add(c, e));
-        r.jy = fma(axis, dy, sub(c, e));
-        r.xy = sub(a, b);
-        r.g = fma(own, o, fma(axis, add(sx, sy), sd));
-    } else {
-        r.xx = sx;
-        r.yy = sy;
-        r.jx = dx;
-        r.jy = dy;
-        r.g = fma(own, o, add(sx, sy));
-    }
-    return r;
-}
 
 // Near contact of the pair (x, y0), (x, y1) in plane z: bit 0 / 1 of the result is
 // set if phi at a probe node, k = 1 .. h_c along n_out = (ax, ay, az), exceeds its
@@ -417,7 +358,7 @@ __device__ __forceinline__ void cg_pair_item(const float* __restrict__ in, float
                 const int nt = (H + st.par) * W + lane, nb = (H + 2 + st.par) * W + lane;
                 emit_plane(c.c, [](int, int cy) { return cy == 1; }, [&](auto dd, float2 c0, float2 c1) {
                     using D = decltype(dd);
-                    constexpr int kt = C::dir(D::cx, 1), kb = C::dir(D::cx, -1);
+                    constexpr int kt = plane_dir(D::cx, 1), kb = plane_dir(D::cx, -1);
                     if constexpr (kC || D::cx == 0) {
                         f4(G4)[4 * (kt * HN + nt)] = c0.x;
                         f4(G4)[4 * (kt * HN + nt) + 2] = c1.x;
@@ -503,7 +444,7 @@ __device__ __forceinline__ void cg_pair_item(const float* __restrict__ in, float
             if (LLB_IN(n1, HN, kChkPublish)) {
                 emit_plane(c.c, [](int, int) { return true; }, [&](auto dd, float2 c0, float2 c1) {
                     using D = decltype(dd);
-                    constexpr int kk = C::dir(D::cx, D::cy);
+                    constexpr int kk = plane_dir(D::cx, D::cy);
                     const int up = (H + st.par) * W + lane, dn = (H + 2 + st.par) * W + lane;
                     if constexpr (kk < C::N4) {
                         G4[kk * HN + n1] = make_float4(c0.x, c0.y, c1.x, c1.y);

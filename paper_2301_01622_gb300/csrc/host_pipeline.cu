@@ -179,7 +179,7 @@ extern "C" int llb_step_host(llb_ctx* c, const void* host_in, void* host_out, in
             }
             if (e == cudaSuccess)
                 e = two ? launch_cg_tiled_range(*c, c->buf[cur], c->buf[1 - cur], zb[k], zb[k + 1], scmp)
-                        : launch_moment_tiled_range(*c, cur, c->buf[cur], c->buf[1 - cur], zb[k], zb[k + 1], scmp);
+                        : launch_moment_tiled_range(*c, cur, c->buf[cur], c->buf[1 - cur], zb[k], zb[k + 1], scmp, copy_out);
             if (copy_out && e == cudaSuccess) {
                 e = launch_shifted_to_canonical_range(*c, c->buf[1 - cur], dev_o, host_dtype, zb[k], zb[k + 1], scmp);
                 if (e == cudaSuccess) e = cudaEventRecord(ev_ready[k], scmp);
@@ -195,7 +195,7 @@ extern "C" int llb_step_host(llb_ctx* c, const void* host_in, void* host_out, in
         // middle steps on the step stream, then the last one with the copies out
         for (int s = 1; s < nsteps - 1 && e == cudaSuccess; ++s) {
             e = two ? launch_cg_tiled_range(*c, c->buf[cur], c->buf[1 - cur], 0, c->nz, scmp)
-                    : launch_moment_tiled_range(*c, cur, c->buf[cur], c->buf[1 - cur], 0, c->nz, scmp);
+                    : launch_moment_tiled_range(*c, cur, c->buf[cur], c->buf[1 - cur], 0, c->nz, scmp, false);
             cur = 1 - cur;
         }
         if (e == cudaSuccess) pipelined_step(false, true);

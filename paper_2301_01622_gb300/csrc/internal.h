@@ -35,7 +35,7 @@ struct llb_ctx {
     CUtensorMap pmap[2];     // TMA L2-prefetch descriptors of buf[0], buf[1] (tiled kernel)
     bool pmap_ok = false;
     void* err_dev = nullptr; // device int: set by a kernel whose bounded wait gave up
-    void* queue_dev = nullptr; // two device ints: work queue of the two-component step, zero between launches
+    void* queue_dev = nullptr; // two device ints: work queue of the pair kernels, zero between launches
     void* buf[2] = {nullptr, nullptr};
     bool owns[2] = {false, false};
     int cur = 0;             // buf[cur] holds the state at time t
@@ -71,10 +71,13 @@ int canonical_fields(const llb_ctx& c);    // 10 or 11
 constexpr int kTiledVariants32 = 6;  // variants of the FP32 tiled kernel (other storage types: 1)
 constexpr int kTmaVariants = 3;      // variants of the TMA kernel
 cudaError_t launch_moment_direct(const llb_ctx& c, const void* in, void* out);
-cudaError_t launch_moment_tiled(const llb_ctx& c, int in_index, const void* in, void* out);
+// ghosts: whether the periodic ghost copies of `out` are needed.  The tiled kernels
+// read none, so of the steps of one call only the last has to write them (kernels
+// that keep them in every step may write them all the same).
+cudaError_t launch_moment_tiled(const llb_ctx& c, int in_index, const void* in, void* out, bool ghosts);
 // Output planes zlo .. zhi-1 only, on stream st (the pipelined host step).
 cudaError_t launch_moment_tiled_range(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi,
-                                      cudaStream_t st);
+                                      cudaStream_t st, bool ghosts);
 cudaError_t launch_moment_tma(const llb_ctx& c, int in_index, void* out);
 int moment_tiled_ctas(const llb_ctx& c);   // persistent grid size, 0 if the kernel cannot run
 int moment_tma_ctas(const llb_ctx& c);
@@ -90,13 +93,13 @@ int moment_tiled_ctas_f64(const llb_ctx& c);
 int moment_tiled_ctas_f16(const llb_ctx& c);
 int moment_tiled_ctas_bf16(const llb_ctx& c);
 cudaError_t launch_moment_tiled_f32(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi,
-                                     cudaStream_t st);
+                                     cudaStream_t st, bool ghosts);
 cudaError_t launch_moment_tiled_f64(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi,
-                                     cudaStream_t st);
+                                     cudaStream_t st, bool ghosts);
 cudaError_t launch_moment_tiled_f16(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi,
-                                     cudaStream_t st);
+                                     cudaStream_t st, bool ghosts);
 cudaError_t launch_moment_tiled_bf16(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi,
-                                     cudaStream_t st);
+                                     cudaStream_t st, bool ghosts);
 void moment_tiled_box_f32(const llb_ctx& c, int* w, int* h);
 void moment_tiled_box_f64(const llb_ctx& c, int* w, int* h);
 void moment_tiled_box_f16(const llb_ctx& c, int* w, int* h);

@@ -14,7 +14,8 @@
 // rows above and below hold periodic ghost copies: columns x = -8..-1 hold
 // x = nx-8..nx-1, columns x = nx..nx+7 hold x = 0..7, rows y = -gy..-1 hold
 // y = ny-gy..ny-1 and rows y = ny..ny+gy-1 hold y = 0..gy-1 (corners
-// likewise), written by every kernel that writes the state.  Whole sectors
+// likewise), written by every kernel that writes the state (of the steps of one
+// call by the last one at least: some kernels read none).  Whole sectors
 // of ghosts are written for the same reason.  With them the tile plus halo a
 // CTA needs is one rectangular box with a 16-byte aligned x start, so one
 // TMA load fetches it without wrapping.

@@ -77,17 +77,17 @@ int moment_tiled_ctas(const llb_ctx& c) {
 }
 
 cudaError_t launch_moment_tiled_range(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi,
-                                      cudaStream_t st) {
+                                      cudaStream_t st, bool ghosts) {
     switch (c.storage) {
-        case LLB_F64: return launch_moment_tiled_f64(c, in_index, in, out, zlo, zhi, st);
-        case LLB_F16S: return launch_moment_tiled_f16(c, in_index, in, out, zlo, zhi, st);
-        case LLB_BF16S: return launch_moment_tiled_bf16(c, in_index, in, out, zlo, zhi, st);
-        default: return launch_moment_tiled_f32(c, in_index, in, out, zlo, zhi, st);
+        case LLB_F64: return launch_moment_tiled_f64(c, in_index, in, out, zlo, zhi, st, ghosts);
+        case LLB_F16S: return launch_moment_tiled_f16(c, in_index, in, out, zlo, zhi, st, ghosts);
+        case LLB_BF16S: return launch_moment_tiled_bf16(c, in_index, in, out, zlo, zhi, st, ghosts);
+        default: return launch_moment_tiled_f32(c, in_index, in, out, zlo, zhi, st, ghosts);
     }
 }
 
-cudaError_t launch_moment_tiled(const llb_ctx& c, int in_index, const void* in, void* out) {
-    return launch_moment_tiled_range(c, in_index, in, out, 0, c.nz, c.stream);
+cudaError_t launch_moment_tiled(const llb_ctx& c, int in_index, const void* in, void* out, bool ghosts) {
+    return launch_moment_tiled_range(c, in_index, in, out, 0, c.nz, c.stream, ghosts);
 }
 
 bool moment_tiled_encode(const llb_ctx& c, void* buf, CUtensorMap* out) {
@@ -98,7 +98,7 @@ bool moment_tiled_encode(const llb_ctx& c, void* buf, CUtensorMap* out) {
         case LLB_BF16S: moment_tiled_box_bf16(c, &w, &h); break;
         default: moment_tiled_box_f32(c, &w, &h); break;
     }
-    return encode_box_map(c, buf, w, h, out);
+    return w > 0 && encode_box_map(c, buf, w, h, out);
 }
 
 LLB_CHK_TU(step)

@@ -22,6 +22,7 @@
 #include <algorithm>
 
 #include "moment_common.cuh"
+#include "moment_pair.cuh"
 
 namespace llb {
 namespace mom {
@@ -244,12 +245,14 @@ struct TiledShape {
     static constexpr int BX = BX_, BY = BY_, MINB = MINB_, OPT = OPT_, PD = PD_;
 };
 
-// FP32 variants (0 = default).  The approximate 1/rho is used by all but
-// variant 2 (measured ~1.5 % faster at 256^3, error far below FP32 storage
+// FP32 variants 1-5 (variant 0 runs two nodes per thread: faster at every size
+// measured, D3Q19 steps of a graph, us: 16^3 3.3 against 3.7 of <64, 4, 2>, 32^3 4.55 /
+// 5.0, 64^3 8.9 / 9.6, 80^3 11.6 / 19.2, 128^3 41 / 48.6, 256^3 267 / 305; D3Q27 32^3
+// 5.5 / 5.6, 64^3 11.0 / 10.9, 80^3 14.2 / 22.2).  The approximate 1/rho is used by all
+// but variant 2 (measured ~1.5 % faster at 256^3, error far below FP32 storage
 // rounding).  The L2 prefetch (variant 1) measured 5 % slower than plain
 // loads on GB300 and is kept for the autotuner.
-constexpr int kTiledVariants = kTiledVariants32;
-template <class T, int V> struct TiledVariant { using type = TiledShape<64, 4, 2, kFastRcp>; };
+template <class T, int V> struct TiledVariant;
 template <> struct TiledVariant<float, 1> { using type = TiledShape<64, 4, 2, kFastRcp | kPrefetch, 2>; };
 template <> struct TiledVariant<float, 2> { using type = TiledShape<64, 4, 2, 0>; };
 template <> struct TiledVariant<float, 3> { using type = TiledShape<64, 8, 1, kFastRcp>; };
@@ -287,12 +290,53 @@ cudaError_t run_tiled_c(const llb_ctx& c, int in_index, const void* in, void* ou
     return cudaGetLastError();
 }
 
-// Box of the L2 prefetch of variant S: the tile plus its halo, widened in x
-// to 16-byte boundaries.
-template <class St, class S>
-void tiled_box(int* w, int* h) {
-    *w = S::BX + 2 * pf_pad<St>();
-    *h = S::BY + 2;
+// Call fn with the one-node shape of the context's variant, or def() where variant 0
+// of FP32 arithmetic runs two nodes per thread (moment_pair.cuh).  VMAX: number of
+// variants the storage offers; a larger number means variant 0.
+template <class T, int VMAX, class F, class D>
+auto with_variant(const llb_ctx& c, F fn, D def) {
+    const int v = c.variant < VMAX ? c.variant : 0;
+    if constexpr (VMAX > 1) {
+        switch (v) {
+            case 1: return fn(typename TiledVariant<T, 1>::type{});
+            case 2: return fn(typename TiledVariant<T, 2>::type{});
+            case 3: return fn(typename TiledVariant<T, 3>::type{});
+            case 4: return fn(typename TiledVariant<T, 4>::type{});
+            case 5: return fn(typename TiledVariant<T, 5>::type{});
+            default: break;
+        }
+    }
+    if constexpr (std::is_same<T, float>::value) return def();
+    else return fn(typename TiledVariant<T, 0>::type{});
+}
+
+template <class L, class T, class St, int VMAX>
+int tiled_ctas(const llb_ctx& c) {
+    return with_variant<T, VMAX>(
+        c, [&](auto shape) { return tiled_ctas_c<L, T, St, decltype(shape)>(c); },
+        [&] { return pair_ctas<L, St>(c); });
+}
+
+template <class L, class T, class St, int VMAX>
+cudaError_t run_tiled(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi, cudaStream_t st,
+                      bool ghosts) {
+    return with_variant<T, VMAX>(
+        c, [&](auto shape) { return run_tiled_c<L, T, St, decltype(shape)>(c, in_index, in, out, zlo, zhi, st); },
+        [&] { return run_pair<L, St>(c, in, out, zlo, zhi, st, ghosts); });
+}
+
+// Box of the L2 prefetch: the tile plus its halo, widened in x to 16-byte
+// boundaries; 0 where the variant prefetches nothing.
+template <class T, class St, int VMAX>
+void tiled_box(const llb_ctx& c, int* w, int* h) {
+    *w = *h = 0;
+    if constexpr (VMAX > 1) {
+        using S = typename TiledVariant<T, 1>::type;
+        if (c.variant == 1) {
+            *w = S::BX + 2 * pf_pad<St>();
+            *h = S::BY + 2;
+        }
+    }
 }
 
 }  // namespace mom
@@ -302,52 +346,14 @@ void tiled_box(int* w, int* h) {
 // type T and storage type St (VMAX: number of variants this storage offers).
 #define LLB_TILED_ENTRY(SUFFIX, T, St, VMAX)                                                                   \
     namespace llb {                                                                                            \
-    namespace {                                                                                                \
-    template <class L>                                                                                         \
-    int ctas_l(const llb_ctx& c) {                                                                             \
-        switch (c.variant < VMAX ? c.variant : 0) {                                                            \
-            case 1: return mom::tiled_ctas_c<L, T, St, typename mom::TiledVariant<T, 1 % VMAX>::type>(c);      \
-            case 2: return mom::tiled_ctas_c<L, T, St, typename mom::TiledVariant<T, 2 % VMAX>::type>(c);      \
-            case 3: return mom::tiled_ctas_c<L, T, St, typename mom::TiledVariant<T, 3 % VMAX>::type>(c);      \
-            case 4: return mom::tiled_ctas_c<L, T, St, typename mom::TiledVariant<T, 4 % VMAX>::type>(c);      \
-            case 5: return mom::tiled_ctas_c<L, T, St, typename mom::TiledVariant<T, 5 % VMAX>::type>(c);      \
-            default: return mom::tiled_ctas_c<L, T, St, typename mom::TiledVariant<T, 0>::type>(c);            \
-        }                                                                                                      \
-    }                                                                                                          \
-    template <class L>                                                                                         \
-    cudaError_t run_l(const llb_ctx& c, int in_index, const void* in, void* out, int zlo, int zhi,         \
-                      cudaStream_t st) {                             \
-        switch (c.variant < VMAX ? c.variant : 0) {                                                            \
-            case 1: return mom::run_tiled_c<L, T, St, typename mom::TiledVariant<T, 1 % VMAX>::type>(c, in_index, in, out, zlo, zhi, st); \
-            case 2: return mom::run_tiled_c<L, T, St, typename mom::TiledVariant<T, 2 % VMAX>::type>(c, in_index, in, out, zlo, zhi, st); \
-            case 3: return mom::run_tiled_c<L, T, St, typename mom::TiledVariant<T, 3 % VMAX>::type>(c, in_index, in, out, zlo, zhi, st); \
-            case 4: return mom::run_tiled_c<L, T, St, typename mom::TiledVariant<T, 4 % VMAX>::type>(c, in_index, in, out, zlo, zhi, st); \
-            case 5: return mom::run_tiled_c<L, T, St, typename mom::TiledVariant<T, 5 % VMAX>::type>(c, in_index, in, out, zlo, zhi, st); \
-            default: return mom::run_tiled_c<L, T, St, typename mom::TiledVariant<T, 0>::type>(c, in_index, in, out, zlo, zhi, st); \
-        }                                                                                                      \
-    }                                                                                                          \
-    template <class L>                                                                                         \
-    void box_l(const llb_ctx& c, int* w, int* h) {                                                             \
-        switch (c.variant < VMAX ? c.variant : 0) {                                                            \
-            case 1: return mom::tiled_box<St, typename mom::TiledVariant<T, 1 % VMAX>::type>(w, h);            \
-            case 2: return mom::tiled_box<St, typename mom::TiledVariant<T, 2 % VMAX>::type>(w, h);            \
-            case 3: return mom::tiled_box<St, typename mom::TiledVariant<T, 3 % VMAX>::type>(w, h);            \
-            case 4: return mom::tiled_box<St, typename mom::TiledVariant<T, 4 % VMAX>::type>(w, h);            \
-            case 5: return mom::tiled_box<St, typename mom::TiledVariant<T, 5 % VMAX>::type>(w, h);            \
-            default: return mom::tiled_box<St, typename mom::TiledVariant<T, 0>::type>(w, h);                  \
-        }                                                                                                      \
-    }                                                                                                          \
-    }                                                                                                          \
     int moment_tiled_ctas_##SUFFIX(const llb_ctx& c) {                                                         \
-        return c.Q == 19 ? ctas_l<D3Q19>(c) : ctas_l<D3Q27>(c);                                                \
+        return c.Q == 19 ? mom::tiled_ctas<D3Q19, T, St, VMAX>(c) : mom::tiled_ctas<D3Q27, T, St, VMAX>(c);    \
     }                                                                                                          \
     cudaError_t launch_moment_tiled_##SUFFIX(const llb_ctx& c, int in_index, const void* in, void* out,        \
-                                             int zlo, int zhi, cudaStream_t st) {                              \
-        return c.Q == 19 ? run_l<D3Q19>(c, in_index, in, out, zlo, zhi, st)                                    \
-                         : run_l<D3Q27>(c, in_index, in, out, zlo, zhi, st);                                   \
+                                             int zlo, int zhi, cudaStream_t st, bool ghosts) {                 \
+        return c.Q == 19 ? mom::run_tiled<D3Q19, T, St, VMAX>(c, in_index, in, out, zlo, zhi, st, ghosts)      \
+                         : mom::run_tiled<D3Q27, T, St, VMAX>(c, in_index, in, out, zlo, zhi, st, ghosts);     \
     }                                                                                                          \
-    void moment_tiled_box_##SUFFIX(const llb_ctx& c, int* w, int* h) {                                         \
-        if (c.Q == 19) box_l<D3Q19>(c, w, h); else box_l<D3Q27>(c, w, h);                                      \
-    }                                                                                                          \
+    void moment_tiled_box_##SUFFIX(const llb_ctx& c, int* w, int* h) { mom::tiled_box<T, St, VMAX>(c, w, h); } \
     LLB_CHK_TU(tiled_##SUFFIX)                                                                                 \
     }
