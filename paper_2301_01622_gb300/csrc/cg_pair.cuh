@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "cg_kernel.cuh"
+#include "overlap.cuh"
 #include "pair_march.cuh"
 #include "tma.cuh"
 
@@ -688,6 +689,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
     // Items from a queue (queue[0]: next item, queue[1]: CTAs done): those that hold an
     // interface take longer.  The last CTA to leave resets it for the next launch.
     __shared__ int s_it;
+    dep_wait();
     for (;;) {
         if (threadIdx.x == 0) s_it = atomicAdd(queue, 1);
         __syncthreads();
@@ -696,6 +698,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         if (it >= sc.nitems) break;
         cg_pair_item<L, H>(in, out, &maps, lay, k, sc, it, zlo, nzr, st, err, budget);
     }
+    dep_launch();
     cg_pair_end<C>(st, bar);
     if (threadIdx.x == 0 && atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {
         queue[0] = 0;

@@ -36,16 +36,17 @@ cudaError_t cg_run_v(const llb_ctx& c, const void* in, void* out, int zlo, int z
         const Sched2 sc = cg_pair_plan(c, zhi - zlo, K::BX, K::BY, grid);
         CgMaps maps;
         if (!cg_pair_maps(c, in, out, &maps)) return cudaErrorInvalidValue;
-        k_cg_pair<L, kPairH, kPairCtas><<<grid, K::NT, K::smem_bytes, st>>>(
-            static_cast<const float*>(in), static_cast<float*>(out), maps, c.lay, pair_constants<L>(c), sc, zlo,
-            zhi - zlo, static_cast<int*>(c.err_dev), static_cast<int*>(c.queue_dev), wait_cycles(c));
+        return launch_overlapped(k_cg_pair<L, kPairH, kPairCtas>, grid, K::NT, K::smem_bytes, st,
+                                 static_cast<const float*>(in), static_cast<float*>(out), maps, c.lay,
+                                 pair_constants<L>(c), sc, zlo, zhi - zlo, static_cast<int*>(c.err_dev),
+                                 static_cast<int*>(c.queue_dev), wait_cycles(c));
     } else {
         using C = CGCfg<L, T, V::BX, V::BY>;
         const Sched2 sc = plan2(c.nx, c.ny, zhi - zlo, V::BX, V::BY, grid);
         k_cg_tiled<L, T, V::BX, V::BY, V::MINB, V::FAST, V::ROLLED><<<grid, C::NT, C::smem_bytes, st>>>(
             static_cast<const T*>(in), static_cast<T*>(out), c.lay, cg_params<T>(c), sc, zlo, zhi - zlo);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
 }
 
 }  // namespace

@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "moment_common.cuh"
+#include "overlap.cuh"
 #include "pair_march.cuh"
 
 namespace llb {
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
     // beyond the first round, queue[1]: CTAs done), asked for when an item begins.  The
     // last CTA to leave resets it for the next launch.
     __shared__ int s_next;
+    dep_wait();
     for (int it = blockIdx.x; it < sc.nitems;) {
         if (threadIdx.x == 0) s_next = (int)gridDim.x + (sc.nitems > (int)gridDim.x ? atomicAdd(queue, 1) : sc.nitems);
         int x0, y0, za, zb;  // outputs za .. zb-1 of the tile at (x0, y0)
@@ -390,6 +392,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         it = s_next;
         __syncthreads();
     }
+    dep_launch();
     if (threadIdx.x == 0 && atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {
         queue[0] = 0;
         queue[1] = 0;
@@ -441,10 +444,9 @@ cudaError_t run_pair(const llb_ctx& c, const void* in, void* out, int zlo, int z
     using K = PairTile<L, kPairH>;
     const int grid = c.tile_ctas > 0 ? c.tile_ctas : 1;
     const Sched sc = pair_plan(c, zhi - zlo, K::BX, K::BY, grid, ghosts);
-    k_moment_pair<L, S, kPairH, kPairCtas><<<grid, K::NT, K::g_bytes, stream>>>(
-        static_cast<const S*>(in), static_cast<S*>(out), c.lay, coll_constants<L, S>(c.omega), sc, zlo, zhi - zlo,
-        ghosts && c.lay.ghosts, static_cast<int*>(c.queue_dev));
-    return cudaGetLastError();
+    return launch_overlapped(k_moment_pair<L, S, kPairH, kPairCtas>, grid, K::NT, K::g_bytes, stream,
+                             static_cast<const S*>(in), static_cast<S*>(out), c.lay, coll_constants<L, S>(c.omega), sc,
+                             zlo, zhi - zlo, (int)(ghosts && c.lay.ghosts), static_cast<int*>(c.queue_dev));
 }
 
 }  // namespace mom
