@@ -321,6 +321,14 @@ LLB_API int llb_state_device(const llb_ctx* ctx, void** dev_ptr, int* dtype, int
 LLB_API int llb_adjoint(llb_ctx* ctx, int nsteps, int every, const void* dev_gfinal, void* dev_ginit, int dtype,
                         double* dtau);
 
+/* The same in device memory of the caller's (256-byte aligned, at least
+ * llb_adjoint_bytes() bytes, free again when the call returns), for callers
+ * that keep a pool: the allocation is 0.1 to 1 ms of a call.  work NULL: as
+ * llb_adjoint. */
+LLB_API int llb_adjoint_bytes(const llb_ctx* ctx, int nsteps, int every, size_t* out);
+LLB_API int llb_adjoint_in(llb_ctx* ctx, int nsteps, int every, const void* dev_gfinal, void* dev_ginit, int dtype,
+                           double* dtau, void* work, size_t work_bytes);
+
 /* ---- batched ensembles ----------------------------------------------
  * Independent two-component boxes of (possibly) different sizes advanced
  * together: each step is ONE persistent launch whose CTAs walk the work

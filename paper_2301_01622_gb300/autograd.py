@@ -27,6 +27,35 @@ def _params(dtype, stream, cg):
     return llb.llb_params_default(storage=storage, stream=stream, ncomp=2, A_h=0.0, **cg)
 
 
+# Device memory of a call (two state copies, and the adjoint's work) comes from torch's
+# allocator up to this size: it keeps the blocks for the next call and gives them back
+# under memory pressure or on torch.cuda.empty_cache().  Allocated and freed by the
+# library they were 2 of the 6 ms of a 128 x 96 x 64, 40-step gradient.  Above it a call
+# takes tens of ms and more, and its memory should not stay behind in a cache.
+_POOLED_BYTES = 1 << 30
+
+
+def _pooled(nbytes, device):
+    """nbytes of device memory from torch's allocator, None where the library should allocate."""
+    if nbytes > _POOLED_BYTES:
+        return None
+    try:
+        return torch.empty(max(nbytes, 1), dtype=torch.uint8, device=device)
+    except torch.cuda.OutOfMemoryError:
+        return None
+
+
+def _create(m, lattice, tau, cg):
+    """A context for moments m on the current stream, and the memory it lives in."""
+    nz, ny, nx = m.shape[1:]
+    p = _params(m.dtype, torch.cuda.current_stream().cuda_stream, cg)
+    n = (llb.llb_state_bytes(nx, ny, nz, lattice, p) + 255) // 256 * 256
+    mem = _pooled(2 * n, m.device)
+    if mem is not None:
+        p.buffers[0], p.buffers[1] = mem.data_ptr(), mem.data_ptr() + n
+    return llb.llb_create(nx, ny, nz, lattice, tau, p), mem
+
+
 class MomentOnlyEvolve(torch.autograd.Function):
     @staticmethod
     def forward(ctx, m0, tau, nsteps: int, lattice: int, every: int, cg):
@@ -34,9 +63,8 @@ class MomentOnlyEvolve(torch.autograd.Function):
         if not m0.is_cuda or m0.dim() != 4 or m0.shape[0] != nf:
             raise ValueError(f"m0 must be a CUDA tensor of shape ({nf}, nz, ny, nx)")
         m0c = m0.detach().contiguous()
-        nz, ny, nx = m0c.shape[1:]
-        stream = torch.cuda.current_stream().cuda_stream
-        c = llb.llb_create(nx, ny, nz, lattice, float(tau), _params(m0c.dtype, stream, cg))
+        tau_value = float(tau)
+        c, mem = _create(m0c, lattice, tau_value, cg)  # mem lives until c is destroyed
         try:
             llb.llb_init_moments_device(c, m0c)
             llb.llb_step(c, nsteps)
@@ -46,20 +74,19 @@ class MomentOnlyEvolve(torch.autograd.Function):
         finally:
             llb.llb_destroy(c)
         ctx.save_for_backward(m0c)
-        ctx.tau, ctx.nsteps, ctx.lattice, ctx.every, ctx.cg = float(tau), nsteps, lattice, every, cg
+        ctx.tau, ctx.nsteps, ctx.lattice, ctx.every, ctx.cg = tau_value, nsteps, lattice, every, cg
         ctx.tau_shape = tau.shape if isinstance(tau, torch.Tensor) else None
         return out
 
     @staticmethod
     def backward(ctx, gout):
         (m0c,) = ctx.saved_tensors
-        nz, ny, nx = m0c.shape[1:]
-        stream = torch.cuda.current_stream().cuda_stream
-        c = llb.llb_create(nx, ny, nz, ctx.lattice, ctx.tau, _params(m0c.dtype, stream, ctx.cg))
+        c, mem = _create(m0c, ctx.lattice, ctx.tau, ctx.cg)
         try:
             llb.llb_init_moments_device(c, m0c)
             ginit = torch.empty_like(m0c)
-            dtau = llb.llb_adjoint(c, ctx.nsteps, gout.to(m0c.dtype).contiguous(), ginit, every=ctx.every)
+            work = _pooled(llb.llb_adjoint_bytes(c, ctx.nsteps, ctx.every), m0c.device)
+            dtau = llb.llb_adjoint(c, ctx.nsteps, gout.to(m0c.dtype).contiguous(), ginit, every=ctx.every, work=work)
         finally:
             llb.llb_destroy(c)
         gtau = None

@@ -761,58 +761,111 @@ LLB_CHK_TU(adjoint)
 
 }  // namespace llb
 
+namespace llb {
+namespace {
+
+// Device memory of one adjoint call, in the order it is laid out (256-byte pieces).
+// Where the step takes any pair of buffers the starting state is the context's own and
+// stays in place, so segment 0 needs no checkpoint and a segment no copy of its first
+// state; the others hold a copy of both.
+struct AdjWork {
+    int K, nseg, nck, nslot;
+    size_t sb, nrows, ck, seg, lamA, lamB, lamG, rows, acc, bytes;
+
+    AdjWork(const llb_ctx& c, int nsteps, int every) {
+        K = every > 0 ? every : (int)std::fmax(1.0, std::round(std::sqrt((double)nsteps)));
+        nseg = nsteps > 0 ? (nsteps + K - 1) / K : 0;
+        const bool direct = any_buffer(c);
+        nck = direct ? std::max(nseg - 1, 0) : nseg;
+        nslot = std::min(K, nsteps) - (direct ? 1 : 0);
+        // rows of dL/domega partial sums: one per block of the one-thread-per-node kernels,
+        // or one per CTA of the tiled first pass (at most 32 per SM)
+        nrows = std::max((size_t)adj_grid(c).x * c.ny * c.nz, (size_t)32 * (c.num_sms > 0 ? c.num_sms : 1));
+        bytes = 0;
+        auto piece = [&](size_t n) {
+            const size_t at = bytes;
+            bytes += (n + 255) / 256 * 256;
+            return at;
+        };
+        sb = (c.state_bytes + 255) / 256 * 256;
+        ck = piece(sb * (size_t)nck);
+        seg = piece(sb * (size_t)std::max(nslot, 0));
+        lamA = piece(sb);
+        lamB = piece(sb);
+        lamG = c.ncomp == 2 ? piece(sb) : lamA;  // cotangent of G (3 fields), two components only
+        rows = piece(nrows * sizeof(double));
+        acc = piece(sizeof(double));
+    }
+};
+
+bool adjoint_takes(const llb_ctx& c, int nsteps) {
+    if (c.in_batch || c.scheme != LLB_SCHEME_MOMENT || (c.storage != LLB_F32 && c.storage != LLB_F64) || nsteps < 0)
+        return false;
+    // two components: differentiable only without the near-contact switch and with the smooth normal
+    return c.ncomp != 2 || (c.params.A_h == 0.0 && c.params.grad_eps > 0.0);
+}
+
+}  // namespace
+}  // namespace llb
+
 extern "C" int llb_adjoint(llb_ctx* c, int nsteps, int every, const void* dev_gfinal, void* dev_ginit, int dtype,
                            double* dtau) {
+    return llb_adjoint_in(c, nsteps, every, dev_gfinal, dev_ginit, dtype, dtau, nullptr, 0);
+}
+
+extern "C" int llb_adjoint_bytes(const llb_ctx* c, int nsteps, int every, size_t* out) {
+    if (!c || !out || !llb::adjoint_takes(*c, nsteps)) return LLB_EINVAL;
+    *out = llb::AdjWork(*c, nsteps, every).bytes;
+    return LLB_OK;
+}
+
+extern "C" int llb_adjoint_in(llb_ctx* c, int nsteps, int every, const void* dev_gfinal, void* dev_ginit, int dtype,
+                              double* dtau, void* work, size_t work_bytes) {
     using namespace llb;
     if (!c) return LLB_EINVAL;
     if (c->sticky != LLB_OK) return LLB_ESTATE;
-    if (c->in_batch || c->scheme != LLB_SCHEME_MOMENT || (c->storage != LLB_F32 && c->storage != LLB_F64) ||
-        nsteps < 0 || !dev_gfinal || !dev_ginit || (dtype != LLB_F64 && dtype != LLB_F32))
+    if (!adjoint_takes(*c, nsteps) || !dev_gfinal || !dev_ginit || (dtype != LLB_F64 && dtype != LLB_F32))
         return LLB_EINVAL;
-    // two components: differentiable only without the near-contact switch and with the smooth normal
     const bool two = c->ncomp == 2;
-    if (two && (c->params.A_h != 0.0 || !(c->params.grad_eps > 0.0))) return LLB_EINVAL;
-    const int K = every > 0 ? every : (int)std::fmax(1.0, std::round(std::sqrt((double)nsteps)));
-    const int nseg = nsteps > 0 ? (nsteps + K - 1) / K : 0;
-    const size_t sb = c->state_bytes;
-    // rows of dL/domega partial sums: one per block of the one-thread-per-node kernels,
-    // or one per CTA of the tiled first pass (at most 32 per SM)
-    const size_t nrows = std::max((size_t)adj_grid(*c).x * c->ny * c->nz, (size_t)32 * (c->num_sms > 0 ? c->num_sms : 1));
-    // scratch: nseg checkpoints, K segment states, two cotangents, omega rows, accumulator
-    std::vector<void*> ptrs;
-    auto grab = [&](size_t bytes) -> void* {
-        void* p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        ptrs.push_back(p);
-        return p;
-    };
-    auto release = [&]() {
-        cudaStreamSynchronize(c->stream);
-        for (void* p : ptrs) cudaFree(p);
+    const AdjWork w(*c, nsteps, every);
+    const int K = w.K, nseg = w.nseg;
+    const size_t sb = w.sb;
+    if (work && (work_bytes < w.bytes || reinterpret_cast<uintptr_t>(work) % 256 != 0)) return LLB_EINVAL;
+    void* own = nullptr;
+    if (!work && cudaMalloc(&own, w.bytes) != cudaSuccess) {
         cudaGetLastError();
-    };
-    char* ck = static_cast<char*>(grab(sb * (size_t)(nseg > 0 ? nseg : 1)));
-    char* seg = static_cast<char*>(grab(sb * (size_t)K));
-    void* lamA = grab(sb);
-    void* lamB = grab(sb);
-    void* lamG = two ? grab(sb) : lamA;  // cotangent of G (3 fields), two components only
-    double* rows = static_cast<double*>(grab(nrows * sizeof(double)));
-    double* acc = static_cast<double*>(grab(sizeof(double)));
-    if (!ck || !seg || !lamA || !lamB || !lamG || !rows || !acc) {
-        release();
         return LLB_ENOMEM;
     }
+    auto release = [&]() {
+        cudaStreamSynchronize(c->stream);
+        if (own) cudaFree(own);
+        cudaGetLastError();
+    };
+    char* const base = static_cast<char*>(work ? work : own);
+    char *const ck = base + w.ck, *const seg = base + w.seg;
+    void *const lamA = base + w.lamA, *const lamB = base + w.lamB, *const lamG = base + w.lamG;
+    double *const rows = reinterpret_cast<double*>(base + w.rows), *const acc = reinterpret_cast<double*>(base + w.acc);
+    const size_t nrows = w.nrows;
     const int cur0 = c->cur;
     const long long t0 = c->t;
     cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(double), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, nrows * sizeof(double), c->stream);
-    // forward with checkpoints (checkpoint k = state at step k K)
-    for (int s = 0; s < nsteps && e == cudaSuccess; ++s) {
+    // State s of the trajectory where the step takes any pair of buffers: the context's
+    // own, a checkpoint (every K steps) or a slot of the segment at hand.
+    const bool direct = any_buffer(*c);
+    auto state = [&](int s) -> char* {
+        if (!direct) return seg + (size_t)(s % K) * sb;
+        if (s == 0) return static_cast<char*>(c->buf[cur0]);
+        return s % K == 0 ? ck + (size_t)(s / K - 1) * sb : seg + (size_t)(s % K - 1) * sb;
+    };
+    // forward to the last state the sweep reads, nsteps - 1: the slots then hold the last segment
+    for (int s = 0; s + 1 < nsteps && e == cudaSuccess && direct; ++s) e = fwd(*c, state(s), state(s + 1));
+    // other steps: in the context's buffers, up to the last checkpoint
+    for (int s = 0; s < nsteps && e == cudaSuccess && !direct; ++s) {
         if (s % K == 0)
-            e = cudaMemcpyAsync(ck + (size_t)(s / K) * sb, c->buf[c->cur], sb, cudaMemcpyDeviceToDevice, c->stream);
+            e = cudaMemcpyAsync(ck + (size_t)(s / K) * sb, c->buf[c->cur], c->state_bytes, cudaMemcpyDeviceToDevice,
+                                c->stream);
+        if (s == (nseg - 1) * K) break;
         if (e == cudaSuccess) e = fwd_one(c);
     }
     // cotangent of the final state
@@ -834,17 +887,12 @@ extern "C" int llb_adjoint(llb_ctx* c, int nsteps, int every, const void* dev_gf
     for (int k = nseg - 1; k >= 0 && e == cudaSuccess; --k) {
         const int s0 = k * K, s1 = s0 + K < nsteps ? s0 + K : nsteps;
         // recompute the states s0 .. s1-1 of this segment from its checkpoint
-        // state s of the segment: the checkpoint itself, then the slots stepped one into the
-        // next (no state is copied), if the step takes any pair of buffers
-        const bool direct = any_buffer(*c);
-        auto state = [&](int s) { return direct && s == s0 ? ck + (size_t)k * sb : seg + (size_t)(s - s0) * sb; };
         if (direct) {
-            for (int s = s0; s + 1 < s1 && e == cudaSuccess; ++s) e = fwd(*c, state(s), state(s + 1));
+            for (int s = s0; s + 1 < s1 && e == cudaSuccess && k < nseg - 1; ++s) e = fwd(*c, state(s), state(s + 1));
         } else {
-            e = cudaMemcpyAsync(c->buf[c->cur], ck + (size_t)k * sb, sb, cudaMemcpyDeviceToDevice, c->stream);
+            e = cudaMemcpyAsync(c->buf[c->cur], ck + (size_t)k * sb, c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
             for (int s = s0; s < s1 && e == cudaSuccess; ++s) {
-                e = cudaMemcpyAsync(seg + (size_t)(s - s0) * sb, c->buf[c->cur], sb, cudaMemcpyDeviceToDevice,
-                                    c->stream);
+                e = cudaMemcpyAsync(state(s), c->buf[c->cur], c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
                 if (e == cudaSuccess && s + 1 < s1) e = fwd_one(c);
             }
         }
@@ -875,7 +923,8 @@ extern "C" int llb_adjoint(llb_ctx* c, int nsteps, int every, const void* dev_gf
     double domega = 0.0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&domega, acc, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     // restore the initial state
-    if (e == cudaSuccess && nseg > 0) e = cudaMemcpyAsync(c->buf[cur0], ck, sb, cudaMemcpyDeviceToDevice, c->stream);
+    if (e == cudaSuccess && nseg > 0 && !direct)
+        e = cudaMemcpyAsync(c->buf[cur0], ck, c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     c->cur = cur0;
     c->t = t0;

@@ -329,8 +329,9 @@ int llb_create(llb_ctx** out, int nx, int ny, int nz, int lattice, double tau, c
         if (cudaMemsetAsync(c->buf[b], 0, bytes, c->stream) != cudaSuccess) { cudaGetLastError(); return bail(LLB_ECUDA); }
     }
     c->diag_scratch_bytes = (size_t)diag_blocks(*c) * 16 * sizeof(double) + 256;
-    if (cudaMalloc(&c->diag_scratch, c->diag_scratch_bytes + sizeof(llb_diag)) != cudaSuccess) { cudaGetLastError(); c->diag_scratch = nullptr; return bail(LLB_ENOMEM); }
-    if (cudaMalloc(&c->flag_dev, 4 * sizeof(int)) != cudaSuccess) { cudaGetLastError(); c->flag_dev = nullptr; return bail(LLB_ENOMEM); }
+    const size_t flag_at = (c->diag_scratch_bytes + sizeof(llb_diag) + 255) / 256 * 256;
+    if (cudaMalloc(&c->diag_scratch, flag_at + 4 * sizeof(int)) != cudaSuccess) { cudaGetLastError(); c->diag_scratch = nullptr; return bail(LLB_ENOMEM); }
+    c->flag_dev = static_cast<char*>(c->diag_scratch) + flag_at;
     c->err_dev = static_cast<int*>(c->flag_dev) + 1;
     c->queue_dev = static_cast<int*>(c->flag_dev) + 2;
     if (c->scheme != LLB_SCHEME_MOMENT && c->ncomp == 2 &&
@@ -369,7 +370,6 @@ void llb_destroy(llb_ctx* c) {
         if (c->owns[b] && c->buf[b]) cudaFree(c->buf[b]);
     if (c->staging) cudaFree(c->staging);
     if (c->diag_scratch) cudaFree(c->diag_scratch);
-    if (c->flag_dev) cudaFree(c->flag_dev);
     if (c->phi_scratch) cudaFree(c->phi_scratch);
     if (c->staging_out) cudaFree(c->staging_out);
     for (int k = 0; k < 3; ++k)

@@ -47,7 +47,7 @@ struct llb_ctx {
     size_t staging_out_bytes = 0;
     cudaStream_t pipe[3] = {nullptr, nullptr, nullptr};  // copy-in, step, copy-out streams of llb_step_host
     size_t diag_scratch_bytes = 0;
-    void* flag_dev = nullptr;      // device int for init-time checks
+    void* flag_dev = nullptr;      // device int for init-time checks (behind diag_scratch, as the next two)
     long long t = 0;
     int sticky = LLB_OK;
     std::string msg;

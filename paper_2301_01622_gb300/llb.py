@@ -92,6 +92,9 @@ _SIGS = {
     "llb_batch_autotune": (C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_int)]),
     "llb_adjoint": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_int,
                               C.POINTER(C.c_double)]),
+    "llb_adjoint_bytes": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.POINTER(C.c_size_t)]),
+    "llb_adjoint_in": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_int,
+                                 C.POINTER(C.c_double), C.c_void_p, C.c_size_t]),
     "llb_checked_status": (C.c_int, [C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_longlong)]),
     "llb_status_string": (C.c_char_p, [C.c_int]),
     "llb_last_error": (C.c_char_p, [C.c_void_p]),
@@ -233,15 +236,24 @@ def llb_autotune(ctx, trials: int = 5):
     return k.value, v.value
 
 
-def llb_adjoint(ctx, nsteps, gfinal_dev, ginit_dev, every: int = 0) -> float:
+def llb_adjoint_bytes(ctx, nsteps, every: int = 0) -> int:
+    out = C.c_size_t()
+    _check(lib().llb_adjoint_bytes(ctx, int(nsteps), int(every), C.byref(out)), "llb_adjoint_bytes", ctx)
+    return int(out.value)
+
+
+def llb_adjoint(ctx, nsteps, gfinal_dev, ginit_dev, every: int = 0, work=None) -> float:
     """Gradient of a loss w.r.t. the initial canonical moments (written into
-    ginit_dev) and tau (returned), given dL/d(final moments) in gfinal_dev."""
+    ginit_dev) and tau (returned), given dL/d(final moments) in gfinal_dev.
+    work: device bytes to work in (at least llb_adjoint_bytes; default: the
+    library allocates them for the call)."""
     dt = _dtype_code(gfinal_dev)
     if _dtype_code(ginit_dev) != dt:
         raise TypeError("gfinal and ginit must have the same dtype")
     dtau = C.c_double()
-    _check(lib().llb_adjoint(ctx, int(nsteps), int(every), _ptr(gfinal_dev), _ptr(ginit_dev), dt, C.byref(dtau)),
-           "llb_adjoint", ctx)
+    _check(lib().llb_adjoint_in(ctx, int(nsteps), int(every), _ptr(gfinal_dev), _ptr(ginit_dev), dt, C.byref(dtau),
+                                _ptr(work) if work is not None else None,
+                                work.numel() * work.element_size() if work is not None else 0), "llb_adjoint", ctx)
     return float(dtau.value)
 
 

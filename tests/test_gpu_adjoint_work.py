@@ -1,0 +1,49 @@
+"""llb_adjoint over the step kernels and its working memory: kernels that take any
+pair of state buffers (states stepped in place) and kernels tied to the context's own
+(states copied) give one gradient and leave the state as it was, in the library's
+memory and in the caller's."""
+import numpy as np
+import pytest
+
+from paper_2301_01622_gb300 import inputs, llb
+
+pytestmark = pytest.mark.gpu
+
+SHAPE = (48, 13, 9)
+CASES = [(llb.LLB_KERNEL_TILED, 0), (llb.LLB_KERNEL_TILED, 1), (llb.LLB_KERNEL_TMA, 2), (llb.LLB_KERNEL_DIRECT, 0)]
+
+
+def _grad(kernel, variant, storage, steps, every, give):
+    import torch
+
+    nx, ny, nz = SHAPE
+    dt = torch.float64 if storage == llb.LLB_F64 else torch.float32
+    m0 = inputs.random_moments(nx, ny, nz, seed=2)
+    g = torch.from_numpy(np.random.default_rng(5).uniform(-1, 1, m0.shape)).to("cuda", dt)
+    gi = torch.empty_like(g)
+    p = llb.llb_params_default(storage=storage, kernel=kernel, variant=variant if storage == llb.LLB_F32 else 0)
+    c = llb.llb_create(nx, ny, nz, 19, 0.8, p)
+    try:
+        llb.llb_init_moments(c, m0)
+        before = llb.llb_get_moments(c, np.empty_like(m0))
+        n = llb.llb_adjoint_bytes(c, steps, every)
+        work = torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda") if give else None
+        dtau = llb.llb_adjoint(c, steps, g, gi, every=every, work=work)
+        assert np.array_equal(before, llb.llb_get_moments(c, np.empty_like(m0)))
+        if give:
+            with pytest.raises(llb.LLBError):
+                llb.llb_adjoint(c, steps, g, gi, every=every, work=work[:n - 1])
+    finally:
+        llb.llb_destroy(c)
+    return gi.double().cpu().numpy(), dtau
+
+
+@pytest.mark.parametrize("storage, tol", [(llb.LLB_F64, 1e-12), (llb.LLB_F32, 1e-5)], ids=["f64", "f32"])
+@pytest.mark.parametrize("steps, every", [(0, 0), (1, 0), (7, 1), (7, 3), (6, 3), (7, 20)])
+def test_step_kernels_and_working_memory(steps, every, storage, tol):
+    ref, rtau = _grad(llb.LLB_KERNEL_DIRECT, 0, llb.LLB_F64, steps, 1, False)
+    for kernel, variant in CASES:
+        for give in (False, True):
+            got, dtau = _grad(kernel, variant, storage, steps, every, give)
+            assert np.abs(got - ref).max() <= tol * np.abs(ref).max(), (kernel, variant, give)
+            assert abs(dtau - rtau) <= 10 * tol * max(abs(rtau), 1.0), (kernel, variant, give)
