@@ -24,9 +24,9 @@
 // lam_rho1(z) and lam_d(z).
 //
 // For two components the first pass (everything but the transposed gradient
-// stencil) runs tiled by default (k_adjoint_cg_tiled, below); one component
-// keeps the one-thread-per-node k_adjoint_step, a plain linear gather whose
-// neighbour loads hit L1 (a tiled form of it measured 13-18 % slower).
+// stencil) runs tiled by default (k_adjoint_cg_tiled, below); one component runs
+// the march of the forward step for FP32 states (Adjoint, below) and the
+// one-thread-per-node k_adjoint_step, a plain linear gather, for FP64.
 //
 // llb_adjoint runs the forward steps once, keeping the state every K steps
 // (moments only), then walks the segments backwards: each segment is
@@ -43,6 +43,7 @@
 #include "lattice.cuh"
 #include "layout.cuh"
 #include "moment_common.cuh"
+#include "moment_pair.cuh"
 #include "twofloat.cuh"
 
 namespace llb {
@@ -167,6 +168,111 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_step(const T* __restric
     }
     add_block_sum<kAdjThreads>(part, domega_rows + ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
+
+// Adjoint of one FP32 step on the march of the step itself (moment_pair.cuh).  A node
+// publishes its s_i = e_i . lam_new, which has the form of the step's populations: a
+// column with s = lam_d - tr lam_A / 3, j = -lam_j (the adjoint pulls from y + c_i) and
+// a = lam_A.  The sums of the pull are the moments sum w_i s_i (1, -c, c c), from which
+// r_i . s_i and J_C^T follow per node.  A thread holds two nodes; loading all ten fields
+// of 19 neighbours per node, as k_adjoint_step does, kept the load pipe busy: 128 x 96 x
+// 64 D3Q19 took 40.7 us a step, now 26.5.
+template <class L>
+struct Adjoint {
+    static constexpr bool kAdjoint = true;
+    const float* m;
+    float om;
+    double* rows;
+
+    struct Sum {  // of the thread's two nodes, on pairs of FP32 numbers (as Wide<float>)
+        float2 h = {0.0f, 0.0f}, l = {0.0f, 0.0f};
+    };
+    // h + l += a, exactly but for the rounding of l
+    static __device__ __forceinline__ void add2(Sum& t, float2 a) {
+        using namespace pk;
+        const float2 s = pk::add(t.h, a), b = sub(s, t.h);
+        t.l = pk::add(t.l, pk::add(sub(t.h, sub(s, b)), sub(a, b)));
+        t.h = s;
+    }
+    // += a (b r - c)
+    static __device__ __forceinline__ void add_term(Sum& t, float2 a, float2 b, float2 r, float2 c) {
+        using namespace pk;
+        const float2 ph = mul(b, r), pl = fma(b, r, mul(-1.0f, ph));
+        Sum s{ph, pl};
+        add2(s, mul(-1.0f, c));
+        const float2 xh = mul(a, s.h), xl = fma(a, s.h, mul(-1.0f, xh));
+        add2(t, xh);
+        t.l = pk::add(t.l, fma(a, s.l, xl));
+    }
+
+    __device__ __forceinline__ pk::Col<float2> column(const float2* v) const {
+        using namespace pk;
+        Col<float2> c;
+        c.s = col_s(v[4], v[5], v[6], v[0]);
+        c.jx = mul(-1.0f, v[1]);
+        c.jy = mul(-1.0f, v[2]);
+        c.jz = mul(-1.0f, v[3]);
+        c.xx = v[4];
+        c.yy = v[5];
+        c.zz = v[6];
+        c.xy = v[7];
+        c.xz = v[8];
+        c.yz = v[9];
+        return c;
+    }
+    __device__ __forceinline__ void load(float* v, size_t e, size_t stride, size_t fs) const {
+        if (!LLB_IN(e + 9 * stride, 10 * fs, kChkLoad)) return;
+#pragma unroll
+        for (int f = 0; f < 10; ++f) v[f] = __ldg(m + e + f * stride);
+    }
+    // r: sums of the pull in, cotangents of the two nodes (state a, b) out
+    __device__ __forceinline__ void finish(float2* r, const float* a, const float* b, bool ok_lo, bool ok_hi,
+                                           Sum& total) const {
+        using namespace pk;
+        constexpr float wh = (float)Shells<L>::w, wl = (float)(Shells<L>::w - (double)wh);
+        float2 q[10];
+#pragma unroll
+        for (int f = 0; f < 10; ++f) q[f] = col_j(wh, wl, r[f]);
+        float2 la[6];
+        const float2 g15 = mul(-1.5f, q[0]);
+#pragma unroll
+        for (int f = 0; f < 3; ++f) la[f] = fma(4.5f, q[4 + f], g15);
+#pragma unroll
+        for (int f = 3; f < 6; ++f) la[f] = mul(9.0f, q[4 + f]);
+        float2 s[10];
+#pragma unroll
+        for (int f = 0; f < 10; ++f) s[f] = make_float2(a[f], b[f]);
+        const float2 one = make_float2(1.0f, 1.0f);
+        const float2 r0 = rcp1p(1.0f, s[0]);
+        const float2 rinv = fma(r0, sub(one, mul(r0, pk::add(one, s[0]))), r0);
+        const float2 jx = s[1], jy = s[2], jz = s[3];
+        const float2 jj[6] = {mul(jx, jx), mul(jy, jy), mul(jz, jz), mul(jx, jy), mul(jx, jz), mul(jy, jz)};
+        float2 dsum = mul(la[0], jj[0]);
+#pragma unroll
+        for (int k = 1; k < 6; ++k) dsum = fma(la[k], jj[k], dsum);
+        const float2 o = mul(om, rinv);
+        const float2 jx2 = pk::add(jx, jx), jy2 = pk::add(jy, jy), jz2 = pk::add(jz, jz);
+        r[0] = sub(q[0], mul(mul(o, rinv), dsum));
+        r[1] = fma(-3.0f, q[1], mul(o, fma(jx2, la[0], fma(jy, la[3], mul(jz, la[4])))));
+        r[2] = fma(-3.0f, q[2], mul(o, fma(jy2, la[1], fma(jx, la[3], mul(jz, la[5])))));
+        r[3] = fma(-3.0f, q[3], mul(o, fma(jz2, la[2], fma(jx, la[4], mul(jy, la[5])))));
+#pragma unroll
+        for (int k = 0; k < 6; ++k) r[4 + k] = mul(1.0f - om, la[k]);
+        // dL/domega: lam'_A : (j j / rho - A)
+        Sum t;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) add_term(t, la[k], jj[k], rinv, s[4 + k]);
+        if (!ok_lo) t.h.x = t.l.x = 0.0f;
+        if (!ok_hi) t.h.y = t.l.y = 0.0f;
+        add2(total, t.h);
+        total.l = pk::add(total.l, t.l);
+    }
+    __device__ __forceinline__ void end(const Sum& total) const {
+        Wide<float> part;
+        part.v = Two{total.h.x, total.l.x};
+        part.v.add(Two{total.h.y, total.l.y});
+        add_block_sum<mom::PairTile<L, mom::kPairH>::NT>(part, rows + blockIdx.x);
+    }
+};
 
 template <class T>
 struct CGAdjPar {
@@ -658,20 +764,40 @@ __global__ void k_cot2_internal_to_canon(const T* __restrict__ lam, void* __rest
 
 dim3 adj_grid(const llb_ctx& c) { return dim3((c.nx + kAdjThreads - 1) / kAdjThreads, c.ny, c.nz); }
 
+// Three CTAs of four warps per SM: 168 registers, of which the pull, two nodes' state and
+// the loads ahead take all (four CTAs: spills).
+constexpr int kAdjCtas = 3;
+
 template <class L, class T>
-cudaError_t adj_step_t(const llb_ctx& c, const void* lam_new, const void* m, void* lam, double* rows) {
-    k_adjoint_step<L, T><<<adj_grid(c), kAdjThreads, 0, c.stream>>>(static_cast<const T*>(lam_new),
-                                                                     static_cast<const T*>(m), static_cast<T*>(lam),
-                                                                     c.lay, (T)c.omega, rows);
-    return cudaGetLastError();
+cudaError_t adj_step_t(const llb_ctx& c, const void* lam_new, const void* m, void* lam, double* rows, size_t* nrows) {
+    if constexpr (std::is_same<T, float>::value) {
+        using K = mom::PairTile<L, mom::kPairH>;
+        auto kern = mom::k_moment_pair<L, float, mom::kPairH, kAdjCtas, Adjoint<L>>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, K::g_bytes);
+        int per_sm = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::NT, K::g_bytes);
+        if (e != cudaSuccess) return e;
+        const int fit = std::max(per_sm, 1) * c.num_sms;
+        const mom::Sched sc = mom::plan(c.nx, c.ny, c.nz, K::BX, K::BY, fit);
+        *nrows = std::min(sc.nitems, fit);
+        return launch_overlapped(kern, (int)*nrows, K::NT, K::g_bytes, c.stream, static_cast<const float*>(lam_new),
+                                 static_cast<float*>(lam), c.lay, Adjoint<L>{static_cast<const float*>(m), (float)c.omega, rows},
+                                 sc, 0, c.nz, 0, static_cast<int*>(nullptr));
+    } else {
+        k_adjoint_step<L, T><<<adj_grid(c), kAdjThreads, 0, c.stream>>>(static_cast<const T*>(lam_new),
+                                                                         static_cast<const T*>(m), static_cast<T*>(lam),
+                                                                         c.lay, (T)c.omega, rows);
+        *nrows = (size_t)adj_grid(c).x * c.ny * c.nz;
+        return cudaGetLastError();
+    }
 }
 
-cudaError_t adj_step(const llb_ctx& c, const void* lam_new, const void* m, void* lam, double* rows) {
+cudaError_t adj_step(const llb_ctx& c, const void* lam_new, const void* m, void* lam, double* rows, size_t* nrows) {
     if (c.Q == 19)
-        return c.storage == LLB_F64 ? adj_step_t<D3Q19, double>(c, lam_new, m, lam, rows)
-                                    : adj_step_t<D3Q19, float>(c, lam_new, m, lam, rows);
-    return c.storage == LLB_F64 ? adj_step_t<D3Q27, double>(c, lam_new, m, lam, rows)
-                                : adj_step_t<D3Q27, float>(c, lam_new, m, lam, rows);
+        return c.storage == LLB_F64 ? adj_step_t<D3Q19, double>(c, lam_new, m, lam, rows, nrows)
+                                    : adj_step_t<D3Q19, float>(c, lam_new, m, lam, rows, nrows);
+    return c.storage == LLB_F64 ? adj_step_t<D3Q27, double>(c, lam_new, m, lam, rows, nrows)
+                                : adj_step_t<D3Q27, float>(c, lam_new, m, lam, rows, nrows);
 }
 
 // CTAs of the tiled first pass for this context (0 if it cannot run).
@@ -898,7 +1024,7 @@ extern "C" int llb_adjoint_in(llb_ctx* c, int nsteps, int every, const void* dev
         }
         for (int s = s1 - 1; s >= s0 && e == cudaSuccess; --s) {
             e = two ? adj_cg_step(*c, lam_in, state(s), lam_out, lamG, rows, &used)
-                    : adj_step(*c, lam_in, state(s), lam_out, rows);
+                    : adj_step(*c, lam_in, state(s), lam_out, rows, &used);
             void* tmp = lam_in;
             lam_in = lam_out;
             lam_out = tmp;

@@ -132,9 +132,19 @@ __device__ __forceinline__ void store_ghosts(S* __restrict__ out, const Layout& 
     }
 }
 
-template <class L, class S, int H, int MINB>
+// What the march computes: the step itself (Step), or the adjoint of a step, whose
+// streaming is the same with the directions reversed (Adjoint, adjoint.cu).
+template <class S>
+struct Step {
+    static constexpr bool kAdjoint = false;
+    CollK k;
+    struct Sum {};
+    __device__ __forceinline__ pk::Col<float2> column(const float2* v) const { return collide_scaled(v, k); }
+};
+
+template <class L, class S, int H, int MINB, class Op>
 __global__ void __launch_bounds__(32 * (H + 1), MINB)
-    k_moment_pair(const S* __restrict__ in, S* __restrict__ out, Layout lay, CollK ck, Sched sc, int zlo, int nzr, int ghosts,
+    k_moment_pair(const S* __restrict__ in, S* __restrict__ out, Layout lay, Op op, Sched sc, int zlo, int nzr, int ghosts,
                   int* queue) {
     using namespace pk;
     using K = PairTile<L, H>;
@@ -165,11 +175,14 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
 
     // Items: the first by block index, the others from a queue (queue[0]: items taken
     // beyond the first round, queue[1]: CTAs done), asked for when an item begins.  The
-    // last CTA to leave resets it for the next launch.
+    // last CTA to leave resets it for the next launch.  The adjoint takes them round-robin,
+    // so that its sum over the nodes has one order.
     __shared__ int s_next;
+    typename Op::Sum total;
     dep_wait();
     for (int it = blockIdx.x; it < sc.nitems;) {
-        if (threadIdx.x == 0) s_next = (int)gridDim.x + (sc.nitems > (int)gridDim.x ? atomicAdd(queue, 1) : sc.nitems);
+        if (threadIdx.x == 0)
+            s_next = Op::kAdjoint ? it + (int)gridDim.x : (int)gridDim.x + (sc.nitems > (int)gridDim.x ? atomicAdd(queue, 1) : sc.nitems);
         int x0, y0, za, zb;  // outputs za .. zb-1 of the tile at (x0, y0)
         sc.item(it, BX, BY, nzr, x0, y0, za, zb);
         za += zlo;
@@ -201,7 +214,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
                 float2 v[10];
 #pragma unroll
                 for (int f = 0; f < 10; ++f) v[f] = widen(a0[f], a1[f]);
-                Col<float2> c = collide_scaled(v, ck);
+                Col<float2> c = op.column(v);
                 if (more) {
                     load(a0, e0 + zo);
                     load(a1, e1 + zo);
@@ -269,7 +282,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
                 float2 v[10];
 #pragma unroll
                 for (int f = 0; f < 10; ++f) v[f] = widen(lo[f], hi[f]);
-                const Col<float2> c = collide_scaled(v, ck);
+                const Col<float2> c = op.column(v);
                 if (more) {
                     load(lo, e_lo + zo);
                     load(hi, e_hi + zo);
@@ -301,6 +314,15 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
                     GZ[n1] = c.zz;
                     if (w == H - 1) FZ[2 * up + 1] = c.zz.x;
                     if (w == 0) FZ[2 * dn] = c.zz.y;
+                }
+            }
+            // the state at the output nodes, for the adjoint
+            S ml[Op::kAdjoint ? 10 : 1], mh[Op::kAdjoint ? 10 : 1];
+            if constexpr (Op::kAdjoint) {
+                if (s > za) {
+                    const size_t zw = (size_t)(s - 1) * plane;
+                    op.load(ml, e_lo + zw, fs, lay.fs);
+                    op.load(mh, e_hi + zw, fs, lay.fs);
                 }
             }
             bar_sync<1, K::NT>();  // the exchange of plane s is complete
@@ -336,18 +358,24 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
                                      G2[3 * HN + nur]);
             }
             float2 r[10];  // plane s - 1 is complete with the c_z = -1 pulls, qt - qc
-            const float third = (float)kCs2;
             const float2 g = sub(qt.g, qc.g), jx = sub(qt.jx, qc.jx), jy = sub(qt.jy, qc.jy);
             r[0] = add(A.g, g);
             r[1] = add(A.jx, jx);
             r[2] = add(A.jy, jy);
             r[3] = sub(zg, g);
-            r[4] = fma(-third, r[0], add(A.xx, sub(qt.xx, qc.xx)));
-            r[5] = fma(-third, r[0], add(A.yy, sub(qt.yy, qc.yy)));
-            r[6] = fma(-third, r[0], add(zg, g));
+            r[4] = add(A.xx, sub(qt.xx, qc.xx));
+            r[5] = add(A.yy, sub(qt.yy, qc.yy));
+            r[6] = add(zg, g);
             r[7] = kC ? add(A.xy, sub(qt.xy, qc.xy)) : A.xy;
             r[8] = sub(zx, jx);
             r[9] = sub(zy, jy);
+            if constexpr (Op::kAdjoint) {
+                if (s > za && (ok_lo || ok_hi)) op.finish(r, ml, mh, ok_lo, ok_hi, total);
+            } else {
+                const float third = (float)kCs2;
+#pragma unroll
+                for (int f = 4; f < 7; ++f) r[f] = fma(-third, r[0], r[f]);
+            }
             if (s > za && (ok_lo || ok_hi)) {
                 S a[10], b[10];
 #pragma unroll
@@ -393,7 +421,8 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         __syncthreads();
     }
     dep_launch();
-    if (threadIdx.x == 0 && atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {
+    if constexpr (Op::kAdjoint) op.end(total);
+    if (!Op::kAdjoint && threadIdx.x == 0 && atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {
         queue[0] = 0;
         queue[1] = 0;
     }
@@ -430,7 +459,7 @@ inline Sched pair_plan(const llb_ctx& c, int nzr, int BX, int BY, int grid, bool
 template <class L, class S>
 int pair_ctas(const llb_ctx& c) {
     using K = PairTile<L, kPairH>;
-    auto kern = k_moment_pair<L, S, kPairH, kPairCtas>;
+    auto kern = k_moment_pair<L, S, kPairH, kPairCtas, Step<S>>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, K::g_bytes) != cudaSuccess) return 0;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::NT, K::g_bytes) != cudaSuccess || per_sm < 1)
@@ -444,9 +473,9 @@ cudaError_t run_pair(const llb_ctx& c, const void* in, void* out, int zlo, int z
     using K = PairTile<L, kPairH>;
     const int grid = c.tile_ctas > 0 ? c.tile_ctas : 1;
     const Sched sc = pair_plan(c, zhi - zlo, K::BX, K::BY, grid, ghosts);
-    return launch_overlapped(k_moment_pair<L, S, kPairH, kPairCtas>, grid, K::NT, K::g_bytes, stream,
-                             static_cast<const S*>(in), static_cast<S*>(out), c.lay, coll_constants<L, S>(c.omega), sc,
-                             zlo, zhi - zlo, (int)(ghosts && c.lay.ghosts), static_cast<int*>(c.queue_dev));
+    return launch_overlapped(k_moment_pair<L, S, kPairH, kPairCtas, Step<S>>, grid, K::NT, K::g_bytes, stream,
+                             static_cast<const S*>(in), static_cast<S*>(out), c.lay,
+                             Step<S>{coll_constants<L, S>(c.omega)}, sc, zlo, zhi - zlo, (int)(ghosts && c.lay.ghosts), static_cast<int*>(c.queue_dev));
 }
 
 }  // namespace mom

@@ -47,3 +47,30 @@ def test_step_kernels_and_working_memory(steps, every, storage, tol):
             got, dtau = _grad(kernel, variant, storage, steps, every, give)
             assert np.abs(got - ref).max() <= tol * np.abs(ref).max(), (kernel, variant, give)
             assert abs(dtau - rtau) <= 10 * tol * max(abs(rtau), 1.0), (kernel, variant, give)
+
+
+@pytest.mark.parametrize("q", [19, 27])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 1), (5, 4, 3), (29, 5, 4), (30, 6, 5), (31, 7, 3), (61, 13, 4)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_fp32_adjoint_tile_edges(shape, q):
+    """The FP32 adjoint (tiles of 30 x 6, two nodes per thread) against the FP64 one
+    (one node per thread), 3 steps.  FP32 bound 1e-5 of the largest entry, as above."""
+    import torch
+
+    nx, ny, nz = shape
+    m0 = inputs.random_moments(nx, ny, nz, seed=4)
+    g64 = torch.from_numpy(np.random.default_rng(6).uniform(-1, 1, m0.shape)).to("cuda")
+    out = []
+    for storage, dt in ((llb.LLB_F64, torch.float64), (llb.LLB_F32, torch.float32)):
+        g = g64.to(dt)
+        gi = torch.empty_like(g)
+        c = llb.llb_create(nx, ny, nz, q, 0.7, llb.llb_params_default(storage=storage))
+        try:
+            llb.llb_init_moments(c, m0)
+            dtau = llb.llb_adjoint(c, 3, g, gi)
+        finally:
+            llb.llb_destroy(c)
+        out.append((gi.double().cpu().numpy(), dtau))
+    (a, ta), (b, tb) = out
+    assert np.abs(a - b).max() <= 1e-5 * np.abs(a).max()
+    assert abs(ta - tb) <= 1e-4 * max(abs(ta), 1.0)
