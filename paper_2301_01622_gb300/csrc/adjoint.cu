@@ -418,29 +418,66 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_cg_local(const T* __res
 
 // Pass 2: the phase-field chain at node z.  G(y) = 3 sum_k w_k c_k phi(y + c_k)
 // transposed gives lam_phi(z) = 3 sum_k w_k c_k . lam_G(z - c_k); phi = 2 rho1 / rho - 1.
+//
+// A thread walks kPhiPlanes planes of one (x, y).  The in-plane sums of a plane serve
+// the three outputs around it, so it loads 9 neighbours per field and plane instead of
+// 27, at addresses formed once.  96^3 D3Q27 FP32: 23 us before, 17.9 now (8 planes
+// 20.6, too few warps for the latency of the loads; 1 plane 19.0).
+constexpr int kPhiX = 32, kPhiY = 4, kPhiPlanes = 3;
+
 template <class L, class T>
-__global__ void __launch_bounds__(kAdjThreads) k_adjoint_cg_phi(const T* __restrict__ m, const T* __restrict__ lam_g,
-                                                                T* __restrict__ lam, Layout lay) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
-    if (x >= lay.nx) return;
-    const size_t fs = lay.fs;
-    T lphi = T(0);
+__global__ void __launch_bounds__(kPhiX * kPhiY) k_adjoint_cg_phi(const T* __restrict__ m, const T* __restrict__ lam_g,
+                                                                  T* __restrict__ lam, Layout lay) {
+    const int x = blockIdx.x * kPhiX + threadIdx.x, y = blockIdx.y * kPhiY + threadIdx.y;
+    if (x >= lay.nx || y >= lay.ny) return;
+    const int za = blockIdx.z * kPhiPlanes, zb = min(za + kPhiPlanes, lay.nz);
+    const size_t fs = lay.fs, plane = (size_t)lay.px * lay.py;
+    constexpr bool kC = L::has(1, 1, 1);
+    constexpr T w1 = T(3.0 * L::w(1, 0, 0)), w2 = T(3.0 * L::w(1, 1, 0)), w3 = kC ? T(3.0 * L::w(1, 1, 1)) : T(0);
+    size_t o[3][3];  // node (x + dx, y + dy) of plane 0 at [dy + 1][dx + 1]
 #pragma unroll
-    for (int cz = -1; cz <= 1; ++cz)
+    for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
-        for (int cy = -1; cy <= 1; ++cy)
+        for (int dx = -1; dx <= 1; ++dx)
+            o[dy + 1][dx + 1] = LLB_CLAMP(lay.at(wrap_idx(x + dx, lay.nx), wrap_idx(y + dy, lay.ny), 0), fs, kChkLoad);
+    // of one plane: c_z = 0 sum, c_z = +-1 sums of the x, y and of the z components, for
+    // lam_phi(z) = 3 sum w c . lam_G(z - c): signs as if c pointed from z to its neighbour
+    struct Sums { T d0, d1, s1; };
+    auto plane_sums = [&](int z) {
+        const size_t zo = (size_t)wrap_idx(z, lay.nz) * plane;
+        T v[3][3][3];
 #pragma unroll
-            for (int cx = -1; cx <= 1; ++cx) {
-                if (!L::has(cx, cy, cz) || (cx == 0 && cy == 0 && cz == 0)) continue;
-                const size_t q = lay.at(wrap_idx(x - cx, lay.nx), wrap_idx(y - cy, lay.ny), wrap_idx(z - cz, lay.nz));
-                lphi += T(3.0 * L::w(cx, cy, cz)) *
-                        (T(cx) * lam_g[q] + T(cy) * lam_g[fs + q] + T(cz) * lam_g[2 * fs + q]);
-            }
-    const size_t i0 = lay.at(x, y, z);
-    const T rinv = T(1) / (T(1) + m[fs + i0]);
-    lam[i0] += lphi * T(2) * rinv;
-    lam[fs + i0] -= lphi * T(2) * m[i0] * rinv * rinv;
+        for (int f = 0; f < 3; ++f)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) v[f][j][i] = __ldg(lam_g + f * fs + o[j][i] + zo);
+        const T ax = v[0][1][2] - v[0][1][0], ay = v[1][2][1] - v[1][0][1];
+        const T xs = (v[0][2][2] - v[0][2][0]) + (v[0][0][2] - v[0][0][0]);
+        const T ys = (v[1][2][2] - v[1][0][2]) + (v[1][2][0] - v[1][0][0]);
+        const T za4 = (v[2][1][0] + v[2][1][2]) + (v[2][0][1] + v[2][2][1]);
+        Sums r;
+        r.d0 = w1 * (ax + ay) + w2 * (xs + ys);
+        r.d1 = w2 * (ax + ay);
+        r.s1 = w1 * v[2][1][1] + w2 * za4;
+        if (kC) {
+            r.d1 += w3 * (xs + ys);
+            r.s1 += w3 * ((v[2][0][0] + v[2][0][2]) + (v[2][2][0] + v[2][2][2]));
+        }
+        return r;
+    };
+    Sums lo = plane_sums(za - 1), mid = plane_sums(za);
+    for (int z = za; z < zb; ++z) {
+        const Sums hi = plane_sums(z + 1);
+        // the neighbour at z - c carries -c of the sums above
+        const T lphi = -(mid.d0 + (lo.d1 + hi.d1) + (hi.s1 - lo.s1));
+        const size_t i0 = LLB_CLAMP(o[1][1] + (size_t)z * plane, fs, kChkStore);
+        const T rinv = T(1) / (T(1) + m[fs + i0]);
+        lam[i0] += lphi * T(2) * rinv;
+        lam[fs + i0] -= lphi * T(2) * m[i0] * rinv * rinv;
+        lo = mid;
+        mid = hi;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -453,16 +490,78 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_cg_phi(const T* __restr
 // publishes them, with t and phi, into a ring of three planes in shared
 // memory; each receiver of the middle plane then reads two values per
 // direction.  Two barriers per plane (published; ring slot free again).
+//
+// Everything the receiver needs is linear in the moments over the directions of s
+// and t (sum w s (1, c, c c) and the same of t), in sum w c t / |c| and in G.  It forms
+// those plane by plane from sums over directions of one weight and only then applies
+// its own fields, where it evaluated the node's populations and their cotangents
+// direction by direction (2160 instructions per node on D3Q27).  Twelve warps per SM
+// (the ring) leave the loads exposed, so each plane is loaded one plane ahead: 96^3
+// D3Q27 FP32 91 us a step before, 71 now (95 without the loads ahead).
 template <class L, class T, int BX, int BY>
 struct AdjTile {
     static constexpr int NT = BX * BY, HX = BX + 2, HY = BY + 2, HN = HX * HY;
-    static constexpr int NF = L::Q + 2;  // Q projections, t, phi
+    static constexpr int NF = L::Q + 2;  // Q projections, (t, phi) of a node side by side
+    static_assert(HN % 2 == 0, "aligned pairs");
     static constexpr int SLOT = NF * HN;  // elements of one plane of the ring
     static constexpr size_t smem_bytes = 3 * (size_t)SLOT * sizeof(T);
     static constexpr int MINB = sizeof(T) == 4 ? 3 : 1;  // CTAs per SM the register budget targets
     static_assert(NT % 32 == 0, "whole warps");
 };
 constexpr int kAdjBX = 32, kAdjBY = 4;
+
+template <class T>
+struct alignas(2 * sizeof(T)) Pair2 {
+    T t, phi;
+};
+
+// Values of a field at the nine nodes of a plane around a node: at the node, at
+// x +- 1, at y +- 1 and at the diagonal ones (1,1) (-1,-1) (1,-1) (-1,1).
+template <class T>
+struct Nine {
+    T o, xp, xm, yp, ym, pp, mm, pm, mp;
+};
+
+// Sums over a plane's directions with weights wo (own column), wa (axes), wd (diagonals).
+template <bool DIAG, class T>
+__device__ __forceinline__ pk::PlaneSum<T> weighted(const Nine<T>& v, T wo, T wa, T wd) {
+    pk::PlaneSum<T> q;
+    const T sx = v.xp + v.xm, sy = v.yp + v.ym;
+    q.g = wo * v.o + wa * (sx + sy);
+    q.jx = wa * (v.xp - v.xm);
+    q.jy = wa * (v.yp - v.ym);
+    q.xx = wa * sx;
+    q.yy = wa * sy;
+    q.xy = T(0);
+    if (DIAG) {
+        const T sp = v.pp + v.mm, sm = v.pm + v.mp, dp = v.pp - v.mm, dm = v.pm - v.mp, sd = sp + sm;
+        q.g += wd * sd;
+        q.jx += wd * (dp + dm);
+        q.jy += wd * (dp - dm);
+        q.xx += wd * sd;
+        q.yy += wd * sd;
+        q.xy = wd * (sp - sm);
+    }
+    return q;
+}
+
+// sum w (1; c; c c) over all directions from the three planes (c_z = -1, 0, 1).
+template <class T>
+struct Sums10 {
+    T g, j[3], a[6];
+    __device__ __forceinline__ Sums10(const pk::PlaneSum<T>& m, const pk::PlaneSum<T>& z, const pk::PlaneSum<T>& p) {
+        a[2] = p.g + m.g;
+        g = z.g + a[2];
+        j[0] = z.jx + (p.jx + m.jx);
+        j[1] = z.jy + (p.jy + m.jy);
+        j[2] = p.g - m.g;
+        a[0] = z.xx + (p.xx + m.xx);
+        a[1] = z.yy + (p.yy + m.yy);
+        a[3] = z.xy + (p.xy + m.xy);
+        a[4] = p.jx - m.jx;
+        a[5] = p.jy - m.jy;
+    }
+};
 
 // Index of direction (cx, cy, cz) in the lattice, enumerated over cz, cy, cx.
 template <class L>
@@ -478,18 +577,25 @@ __host__ __device__ constexpr int dir_index(int cx, int cy, int cz) {
     return -1;
 }
 
-// Publish node j of the tile-plus-halo region (plane index zq, wrapped) into slot S.
-template <class L, class T, int HN>
-__device__ __forceinline__ void adj_publish(const T* __restrict__ lam_new, const T* __restrict__ m, const Layout& lay,
-                                            size_t i, int j, T* __restrict__ S) {
-    const size_t fs = lay.fs;
-    if (!LLB_IN(i, fs, kChkLoad) || !LLB_IN(j, HN, kChkPublish)) return;
-    T v[11];
+// What a region node publishes from: its 11 cotangents, rho1 and d.
+template <class T>
+struct AdjNode {
+    T v[11], r1, d;
+    __device__ __forceinline__ void load(const T* __restrict__ lam_new, const T* __restrict__ m, size_t i, size_t fs) {
+        if (!LLB_IN(i, fs, kChkLoad)) return;
 #pragma unroll
-    for (int f = 0; f < 11; ++f) v[f] = lam_new[f * fs + i];
-    const T r1 = m[i], d = m[fs + i];
-    S[(L::Q + 1) * HN + j] = T(2) * r1 / (T(1) + d) - T(1);
-    S[L::Q * HN + j] = v[0];
+        for (int f = 0; f < 11; ++f) v[f] = __ldg(lam_new + f * fs + i);
+        r1 = __ldg(m + i);
+        d = __ldg(m + fs + i);
+    }
+};
+
+// Publish node j of the tile-plus-halo region into slot S.
+template <class L, class T, int HN>
+__device__ __forceinline__ void adj_publish(const AdjNode<T>& a, int j, T* __restrict__ S) {
+    if (!LLB_IN(j, HN, kChkPublish)) return;
+    const T* const v = a.v;
+    *reinterpret_cast<Pair2<T>*>(S + L::Q * HN + 2 * j) = Pair2<T>{v[0], T(2) * a.r1 / (T(1) + a.d) - T(1)};
     // s(+-c) = even +- odd, even = v1 + (cc - cs^2 I) : vP, odd = c . vj
     const T ev0 = v[1] - T(kCs2) * (v[5] + v[6] + v[7]);
     S[dir_index<L>(0, 0, 0) * HN + j] = ev0;
@@ -529,23 +635,66 @@ __device__ __forceinline__ void adj_receive(Wide<T>& part, const T* __restrict__
     constexpr int Q = L::Q;
     const T r1 = s[0], d = s[1], jx = s[2], jy = s[3], jz = s[4];
     const T* A = s + 5;  // xx, yy, zz, xy, xz, yz
-    T G[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int cz = -1; cz <= 1; ++cz)
-#pragma unroll
-        for (int cy = -1; cy <= 1; ++cy)
-#pragma unroll
-            for (int cx = -1; cx <= 1; ++cx) {
-                if (!L::has(cx, cy, cz) || (cx == 0 && cy == 0 && cz == 0)) continue;
-                const T* P = cz > 0 ? Sp : (cz < 0 ? Sm : S0);
-                const T wp = T(3.0 * L::w(cx, cy, cz)) * P[(Q + 1) * HN + n + cy * HX + cx];
-                G[0] += T(cx) * wp;
-                G[1] += T(cy) * wp;
-                G[2] += T(cz) * wp;
-            }
+    constexpr bool kC = L::has(1, 1, 1);
+    constexpr T w0 = T(L::w(0, 0, 0)), w1 = T(L::w(1, 0, 0)), w2 = T(L::w(1, 1, 0)), w3 = kC ? T(L::w(1, 1, 1)) : T(0);
+    // moments of s: the projection along c of the neighbour at y + c
+    auto s9 = [&](const T* P, auto czc) {
+        constexpr int cz = decltype(czc)::value;
+        auto at = [&](auto cxc, auto cyc) -> T {
+            constexpr int cx = decltype(cxc)::value, cy = decltype(cyc)::value;
+            if constexpr (L::has(cx, cy, cz)) return P[dir_index<L>(cx, cy, cz) * HN + n + cy * HX + cx];
+            else return T(0);
+        };
+        constexpr std::integral_constant<int, 0> o{};
+        constexpr std::integral_constant<int, 1> p1{};
+        constexpr std::integral_constant<int, -1> m1{};
+        return Nine<T>{at(o, o), at(p1, o), at(m1, o), at(o, p1), at(o, m1), at(p1, p1), at(m1, m1), at(p1, m1), at(m1, p1)};
+    };
+    const Sums10<T> S(weighted<kC>(s9(Sm, std::integral_constant<int, -1>{}), w1, w2, w3),
+                      weighted<true>(s9(S0, std::integral_constant<int, 0>{}), w0, w1, w2),
+                      weighted<kC>(s9(Sp, std::integral_constant<int, 1>{}), w1, w2, w3));
+    // moments of t, K = sum w c t / |c| and G = 3 sum w c phi
+    auto t9 = [&](const T* P, Nine<T>& t, Nine<T>& f) {
+        const Pair2<T>* const q = reinterpret_cast<const Pair2<T>*>(P + Q * HN) + n;
+        auto rd = [&](int off, T& a, T& b) {
+            const Pair2<T> v = q[off];
+            a = v.t;
+            b = v.phi;
+        };
+        rd(0, t.o, f.o);
+        rd(1, t.xp, f.xp);
+        rd(-1, t.xm, f.xm);
+        rd(HX, t.yp, f.yp);
+        rd(-HX, t.ym, f.ym);
+        rd(HX + 1, t.pp, f.pp);
+        rd(-HX - 1, t.mm, f.mm);
+        rd(1 - HX, t.pm, f.pm);
+        rd(HX - 1, t.mp, f.mp);
+    };
+    constexpr T k1 = T(L::w(1, 0, 0)), k2 = T(L::w(1, 1, 0) * inv_len_c(1, 1, 0)),
+                k3 = kC ? T(L::w(1, 1, 1) * inv_len_c(1, 1, 1)) : T(0);
+    T K[3], G[3];
+    Nine<T> tv, fv;
+    t9(Sm, tv, fv);
+    const pk::PlaneSum<T> tm = weighted<kC>(tv, w1, w2, w3), fm = weighted<kC>(fv, w1, w2, w3),
+                          km = weighted<kC>(tv, k1, k2, k3);
+    t9(Sp, tv, fv);
+    const pk::PlaneSum<T> tp = weighted<kC>(tv, w1, w2, w3), fp = weighted<kC>(fv, w1, w2, w3),
+                          kp = weighted<kC>(tv, k1, k2, k3);
+    t9(S0, tv, fv);
+    const pk::PlaneSum<T> tz = weighted<true>(tv, w0, w1, w2), fz = weighted<true>(fv, T(0), w1, w2),
+                          kz = weighted<true>(tv, T(0), k1, k2);
+    const Sums10<T> M(tm, tz, tp);
+    K[0] = kz.jx + (kp.jx + km.jx);
+    K[1] = kz.jy + (kp.jy + km.jy);
+    K[2] = kp.g - km.g;
+    G[0] = T(3) * (fz.jx + (fp.jx + fm.jx));
+    G[1] = T(3) * (fz.jy + (fp.jy + fm.jy));
+    G[2] = T(3) * (fp.g - fm.g);
     const T rho = T(1) + d, rinv = T(1) / rho, om = p.omega;
     const T gn = sqrt(G[0] * G[0] + G[1] * G[1] + G[2] * G[2] + p.eps2);
-    const T nv[3] = {G[0] / gn, G[1] / gn, G[2] / gn};
+    const T ign = T(1) / gn;
+    const T nv[3] = {G[0] * ign, G[1] * ign, G[2] * ign};
     const T ks = p.A_s * gn * T(1.0 / 9.0);
     const T jj[6] = {jx * jx, jy * jy, jz * jz, jx * jy, jx * jz, jy * jz};
     const T nn[6] = {nv[0] * nv[0], nv[1] * nv[1], nv[2] * nv[2], nv[0] * nv[1], nv[0] * nv[2], nv[1] * nv[2]};
@@ -555,50 +704,22 @@ __device__ __forceinline__ void adj_receive(Wide<T>& part, const T* __restrict__
     const T s0 = d - T(1.5) * (Ap[0] + Ap[1] + Ap[2]);
     const T r1r = r1 * rinv;
     const T e = p.beta * r1 * (rho - r1) * rinv;
-    T ld = T(0), lj[3] = {T(0), T(0), T(0)}, la[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    T l_r1r = T(0), l_e = T(0), ln[3] = {T(0), T(0), T(0)};
+    // g'_i + w_i = w_i (1 + s0 + 3 c.j + 4.5 c c : A') summed over the directions with t
+    T l_r1r = (T(1) + s0) * M.g + T(3) * (jx * M.j[0] + jy * M.j[1] + jz * M.j[2]);
+    T l_e = T(0), ln[3], lj[3], la[6];
 #pragma unroll
-    for (int cz = -1; cz <= 1; ++cz)
+    for (int a = 0; a < 3; ++a) {
+        l_r1r += T(4.5) * Ap[a] * M.a[a] + T(9) * Ap[3 + a] * M.a[3 + a];
+        l_e += nv[a] * K[a];
+        ln[a] = e * K[a];
+    }
+    const T ld = S.g + r1r * M.g;
 #pragma unroll
-        for (int cy = -1; cy <= 1; ++cy)
-#pragma unroll
-            for (int cx = -1; cx <= 1; ++cx) {
-                if (!L::has(cx, cy, cz)) continue;
-                const T* P = cz > 0 ? Sp : (cz < 0 ? Sm : S0);
-                const int o = n + cy * HX + cx;
-                const T si = P[dir_index<L>(cx, cy, cz) * HN + o];
-                const T ti = P[Q * HN + o];
-                const T w = T(L::w(cx, cy, cz));
-                T qd = s0;
-                if (cx) qd += T(4.5) * Ap[0];
-                if (cy) qd += T(4.5) * Ap[1];
-                if (cz) qd += T(4.5) * Ap[2];
-                if (cx * cy) qd += T(9 * cx * cy) * Ap[3];
-                if (cx * cz) qd += T(9 * cx * cz) * Ap[4];
-                if (cy * cz) qd += T(9 * cy * cz) * Ap[5];
-                const T gi = w * (qd + T(3 * cx) * jx + T(3 * cy) * jy + T(3 * cz) * jz);
-                l_r1r += ti * (w + gi);
-                if (cx || cy || cz) {
-                    const T il = T(inv_len_c(cx, cy, cz));
-                    const T cn = T(cx) * nv[0] + T(cy) * nv[1] + T(cz) * nv[2];
-                    l_e += ti * w * cn * il;
-                    const T f = ti * e * w * il;
-                    ln[0] += f * T(cx);
-                    ln[1] += f * T(cy);
-                    ln[2] += f * T(cz);
-                }
-                const T ws = w * (si + ti * r1r);
-                ld += ws;
-                lj[0] += T(3 * cx) * ws;
-                lj[1] += T(3 * cy) * ws;
-                lj[2] += T(3 * cz) * ws;
-                la[0] += (T(4.5 * cx * cx) - T(1.5)) * ws;
-                la[1] += (T(4.5 * cy * cy) - T(1.5)) * ws;
-                la[2] += (T(4.5 * cz * cz) - T(1.5)) * ws;
-                la[3] += T(9 * cx * cy) * ws;
-                la[4] += T(9 * cx * cz) * ws;
-                la[5] += T(9 * cy * cz) * ws;
-            }
+    for (int a = 0; a < 3; ++a) {
+        lj[a] = T(3) * (S.j[a] + r1r * M.j[a]);
+        la[a] = T(4.5) * (S.a[a] + r1r * M.a[a]) - T(1.5) * ld;
+        la[3 + a] = T(9) * (S.a[3 + a] + r1r * M.a[3 + a]);
+    }
     T l_rinv = T(0), l_ks = T(0);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
@@ -614,14 +735,14 @@ __device__ __forceinline__ void adj_receive(Wide<T>& part, const T* __restrict__
     ln[0] += ks * (T(2) * nv[0] * la[0] + nv[1] * la[3] + nv[2] * la[4]);
     ln[1] += ks * (T(2) * nv[1] * la[1] + nv[0] * la[3] + nv[2] * la[5]);
     ln[2] += ks * (T(2) * nv[2] * la[2] + nv[0] * la[4] + nv[1] * la[5]);
-    const T l_gn = p.A_s * T(1.0 / 9.0) * l_ks - (ln[0] * G[0] + ln[1] * G[1] + ln[2] * G[2]) / (gn * gn);
+    const T l_gn = p.A_s * T(1.0 / 9.0) * l_ks - (ln[0] * nv[0] + ln[1] * nv[1] + ln[2] * nv[2]) * ign;
     l_rinv += l_r1r * r1 - l_e * p.beta * r1 * r1;
     out[0] = l_r1r * rinv + l_e * p.beta * (T(1) - T(2) * r1 * rinv);
     out[1] = ld - l_rinv * rinv * rinv;
 #pragma unroll
     for (int f = 0; f < 11; ++f) lam[f * fs + i0] = out[f];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) lam_g[a * fs + i0] = ln[a] / gn + l_gn * G[a] / gn;
+    for (int a = 0; a < 3; ++a) lam_g[a * fs + i0] = ln[a] * ign + l_gn * nv[a];
     for (int k = 0; k < 6; ++k) part.add_term(la[k], jj[k], rinv, A[k]);
 }
 
@@ -651,16 +772,26 @@ __global__ void __launch_bounds__(BX * BY, (AdjTile<L, T, BX, BY>::MINB))
         const bool ok = ox < nx && oy < ny;
         const size_t own = ok ? lay.at(ox, oy, 0) : 0;
         auto slot = [&](int q) { return ring + (size_t)((q - za + 1) % 3) * SLOT; };  // q >= za - 1
+        // a plane is loaded while the one before it is received
+        AdjNode<T> a0, a1;
+        auto load = [&](int q) {
+            const size_t zo = (size_t)mom::pmod(q, nz) * plane;
+            a0.load(lam_new, m, off0 + zo, fs);
+            if (j1 < HN) a1.load(lam_new, m, off1 + zo, fs);
+        };
         auto publish = [&](int q) {
             T* S = slot(q);
-            const size_t zo = (size_t)mom::pmod(q, nz) * plane;
-            adj_publish<L, T, HN>(lam_new, m, lay, off0 + zo, t, S);
-            if (j1 < HN) adj_publish<L, T, HN>(lam_new, m, lay, off1 + zo, j1, S);
+            adj_publish<L, T, HN>(a0, t, S);
+            if (j1 < HN) adj_publish<L, T, HN>(a1, j1, S);
         };
+        load(za - 1);
         publish(za - 1);
+        load(za);
         publish(za);
+        load(za + 1);
         for (int q = za; q < zb; ++q) {  // receivers of plane q
             publish(q + 1);
+            if (q + 2 <= zb) load(q + 2);
             T sv[11];
             const size_t iy = own + (size_t)mom::pmod(q, nz) * plane;
             if (ok && LLB_IN(iy, fs, kChkLoad)) {
@@ -839,9 +970,10 @@ cudaError_t adj_cg_step_t(const llb_ctx& c, const void* lam_new, const void* m, 
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_adjoint_cg_phi<L, T><<<adj_grid(c), kAdjThreads, 0, c.stream>>>(static_cast<const T*>(m),
-                                                                       static_cast<const T*>(lam_g),
-                                                                       static_cast<T*>(lam), c.lay);
+    const dim3 phi_grid((c.nx + kPhiX - 1) / kPhiX, (c.ny + kPhiY - 1) / kPhiY, (c.nz + kPhiPlanes - 1) / kPhiPlanes);
+    k_adjoint_cg_phi<L, T><<<phi_grid, dim3(kPhiX, kPhiY), 0, c.stream>>>(static_cast<const T*>(m),
+                                                                      static_cast<const T*>(lam_g),
+                                                                      static_cast<T*>(lam), c.lay);
     return cudaGetLastError();
 }
 

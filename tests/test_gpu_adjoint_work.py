@@ -74,3 +74,30 @@ def test_fp32_adjoint_tile_edges(shape, q):
     (a, ta), (b, tb) = out
     assert np.abs(a - b).max() <= 1e-5 * np.abs(a).max()
     assert abs(ta - tb) <= 1e-4 * max(abs(ta), 1.0)
+
+
+@pytest.mark.parametrize("q", [19, 27])
+@pytest.mark.parametrize("shape", [(4, 4, 4), (33, 5, 7), (32, 8, 4), (31, 9, 8)], ids=lambda s: "x".join(map(str, s)))
+def test_two_component_adjoint_does_not_see_the_tiles(shape, q):
+    """A box shifted along its diagonal has the shifted gradient: where tiles and runs of
+    planes begin must not show.  FP64, 2 steps: 1e-11 of the largest entry (the sums of
+    a node are the same, in another order)."""
+    import torch
+
+    nx, ny, nz = shape
+    m0 = inputs.random_moments(nx, ny, nz, seed=8, nfields=11)
+    g0 = np.random.default_rng(9).uniform(-1, 1, m0.shape)
+    c = llb.llb_create(nx, ny, nz, q, 0.9, llb.llb_params_default(storage=llb.LLB_F64, ncomp=2, grad_eps=0.05))
+    out = []
+    try:
+        for shift in ((0, 0, 0), (1, 2, 3)):
+            g = torch.from_numpy(np.ascontiguousarray(np.roll(g0, shift, axis=(1, 2, 3)))).cuda()
+            gi = torch.empty_like(g)
+            llb.llb_init_moments(c, np.ascontiguousarray(np.roll(m0, shift, axis=(1, 2, 3))))
+            dtau = llb.llb_adjoint(c, 2, g, gi)
+            out.append((np.roll(gi.cpu().numpy(), [-s for s in shift], axis=(1, 2, 3)), dtau))
+    finally:
+        llb.llb_destroy(c)
+    (a, ta), (b, tb) = out
+    assert np.abs(a - b).max() <= 1e-11 * np.abs(a).max()
+    assert abs(ta - tb) <= 1e-10 * max(abs(ta), 1.0)
