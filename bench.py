@@ -174,8 +174,8 @@ def measured_peaks():
     return 6800.0, "fallback (6.8 TB/s)"
 
 
-KERNEL_SOURCES = ("moment_tiled.cuh", "moment_common.cuh", "moment_tiled_f32.cu", "lattice.cuh", "layout.cuh",
-                  "storage.cuh")
+KERNEL_SOURCES = ("moment_pair.cuh", "pair_march.cuh", "packed.cuh", "overlap.cuh", "moment_tiled.cuh",
+                  "moment_common.cuh", "moment_tiled_f32.cu", "lattice.cuh", "layout.cuh", "storage.cuh")
 
 
 def kernel_source_sha():
@@ -673,7 +673,8 @@ def main():
             "frac_of_nominal_7900": main_r["achieved_gbs"] / 7900.0,
             "peak_source": peak_src + ", burst copy figure (the step kernel is timed alone)",
             "algorithmic_bytes_per_launch": main_r["bytes_per_node"] * nodes,
-            "kernel": {1: "k_moment_direct", 2: "k_moment_tiled", 3: "k_moment_tma"}.get(main_r["kernel"], "?") + "<D3Q19,float>", "avg_launch_ms": main_r["launch_ms"]}
+            "kernel": {1: "k_moment_direct", 2: "k_moment_tiled" if args.variant else "k_moment_pair",
+                       3: "k_moment_tma"}.get(main_r["kernel"], "?") + "<D3Q19,float>", "avg_launch_ms": main_r["launch_ms"]}
     line = {
         "metric": METRIC, "value": main_r["mlups"], "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": main_r["ms_per_step"], "higher_is_better": True,

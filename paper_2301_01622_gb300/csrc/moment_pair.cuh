@@ -3,8 +3,8 @@
 //
 // The march of moment_tiled.cuh with the work of a thread doubled.  The one-node
 // form executed 334 thread-instructions per node on D3Q19 at half the issue rate,
-// with 4.4 of 8 warps colliding a halo node per plane; the pair executes about
-// 190 and a CTA's halo is one warp.
+// with 4.4 of 8 warps colliding a halo node per plane; the pair executes
+// 202 and a CTA's halo is one warp.
 //
 // A CTA is H tile warps and a halo warp for the rows above and below.  A warp
 // holds 32 columns, the inner 30 its outputs: the outer two are collided for
