@@ -62,6 +62,16 @@ struct FieldMap {
     }
 };
 
+// Elements from a field of node (x, y, z) to the same field of its ghost copy in x, in
+// a box at least 2 kGhostX wide (a node has one such copy at most); 0 if it has none.
+// 64 bits: in the interleaved state the distance is about ten times nx.
+template <class S, int NF>
+__host__ __device__ __forceinline__ std::ptrdiff_t ghost_shift_x(const Layout& L, int x) {
+    const int copy = x < kGhostX ? x + L.nx : x >= L.nx - kGhostX ? x - L.nx : x;
+    return (std::ptrdiff_t)FieldMap<S, NF>::at(L.at(copy, 0, 0), 0, L.fs) -
+           (std::ptrdiff_t)FieldMap<S, NF>::at(L.at(x, 0, 0), 0, L.fs);
+}
+
 // row_align: multiple the padded row pitch is rounded up to (8; 32 for the
 // interleaved one-component FP32 state).
 inline Layout make_layout(int nx, int ny, int nz, bool padded, int ghost_rows = 1, int row_align = 8) {

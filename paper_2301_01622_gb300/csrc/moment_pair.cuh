@@ -259,9 +259,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         // row), at distances that are the same in every plane and, in x, every row;
         // smaller boxes take the general store_ghosts.
         const bool gsmall = nx < 2 * kGhostX || ny < 2;
-        const int gsx = ox < kGhostX ? nx : ox >= nx - kGhostX ? -nx : 0;
-        const int gdx = gsx ? (int)(FieldMap<S, 10>::at(lay.at(ox + gsx, 0, 0), 0, lay.fs) -
-                                    FieldMap<S, 10>::at(lay.at(ox, 0, 0), 0, lay.fs)) : 0;
+        const std::ptrdiff_t gdx = ok_x ? ghost_shift_x<S, 10>(lay, ox) : 0;
         const bool gy = oy < lay.yo || oy >= ny - lay.yo || oy + H >= ny - lay.yo;  // a row with a copy, warp-uniform
         S lo[10], hi[10];
         load(lo, e_lo + zo);
@@ -390,8 +388,8 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
                 if (ok_lo) store(e_lo + zw, a);
                 if (ok_hi) store(e_hi + zw, b);
                 if (ghosts && gdx && !gsmall) {
-                    if (ok_lo) store(e_lo + zw + gdx, a);
-                    if (ok_hi) store(e_hi + zw + gdx, b);
+                    if (ok_lo) store(e_lo + zw + (size_t)gdx, a);
+                    if (ok_hi) store(e_hi + zw + (size_t)gdx, b);
                 }
                 if (ghosts && (gy || gsmall)) {
                     if (ok_lo) store_ghosts(out, lay, ox, oy, s - 1, a, !gsmall);
