@@ -259,9 +259,11 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         // row), at distances that are the same in every plane and, in x, every row;
         // smaller boxes take the general store_ghosts.
         const bool gsmall = nx < 2 * kGhostX || ny < 2;
-        // (+-nx in a field-major state, where 64 bits cost a spilled register on D3Q27)
-        using Shift = typename std::conditional<IL, std::ptrdiff_t, int>::type;
-        const Shift gdx = !ok_x ? 0 : (Shift)ghost_shift_x<S, 10>(lay, ox);
+        // (+-nx in a field-major state, where 64 bits cost spilled registers on D3Q27)
+        const auto gdx = [&] {
+            if constexpr (IL) return ok_x ? ghost_shift_x<S, 10>(lay, ox) : std::ptrdiff_t(0);
+            else return ox < kGhostX ? nx : ox >= nx - kGhostX ? -nx : 0;
+        }();
         const bool gy = oy < lay.yo || oy >= ny - lay.yo || oy + H >= ny - lay.yo;  // a row with a copy, warp-uniform
         S lo[10], hi[10];
         load(lo, e_lo + zo);
