@@ -222,7 +222,7 @@ struct Adjoint {
     __device__ __forceinline__ void load(float* v, size_t e, size_t stride, size_t fs) const {
         if (!LLB_IN(e + 9 * stride, 10 * fs, kChkLoad)) return;
 #pragma unroll
-        for (int f = 0; f < 10; ++f) v[f] = __ldg(m + e + f * stride);
+        for (int f = 0; f < 10; ++f) v[f] = load_dep(m + e + f * stride);
     }
     // r: sums of the pull in, cotangents of the two nodes (state a, b) out
     __device__ __forceinline__ void finish(float2* r, const float* a, const float* b, bool ok_lo, bool ok_hi,

@@ -215,9 +215,9 @@ struct CgTile {
 // own phi0 by kPhiRise (want: bits to test).  The probes of both nodes are loaded
 // three at a time, so that the step waits for memory once and not per probe; out
 // of line, off the path of the nodes away from interfaces.
-static __device__ __noinline__ int near_contact(const float* __restrict__ r1, const float* __restrict__ dd, int nx,
-                                                int ny, int nz, int px, size_t plane, int x, int y0, int y1, int z,
-                                                int h_c, int want, float2 ax, float2 ay, float2 az, float2 phi0) {
+static __device__ __noinline__ int near_contact(const float* r1, const float* dd, int nx, int ny, int nz, int px,
+                                                size_t plane, int x, int y0, int y1, int z, int h_c, int want,
+                                                float2 ax, float2 ay, float2 az, float2 phi0) {
     // r1, dd: the fields at node (0, 0, 0); a box of at least 8 nodes wraps a probe at most once
     auto wrap = [](int v, int n) { return n >= 8 ? wrap_idx(v, n) : pmod2(v, n); };
     int got = 0;
@@ -238,8 +238,8 @@ static __device__ __noinline__ int near_contact(const float* __restrict__ r1, co
                 const int gz = wrap(z + __float2int_rn(q * bz), nz);
                 const size_t i = gz * plane + (unsigned)(gy * px + gx);
                 const bool in_range = LLB_IN(i + 2 * px + kGhostX, plane * nz, kChkProbe);
-                r[j] = in_range ? __ldg(r1 + i) : 0.0f;
-                d[j] = in_range ? __ldg(dd + i) : 0.0f;
+                r[j] = in_range ? load_dep(r1 + i) : 0.0f;
+                d[j] = in_range ? load_dep(dd + i) : 0.0f;
             }
 #pragma unroll
             for (int j = 0; j < 3; ++j) near |= 2.0f * r[j] > t * (1.0f + d[j]);  // phi = 2 rho1 / rho - 1 > phi0 + rise
@@ -263,10 +263,9 @@ struct March {
 // step publishes); it is loaded two steps ahead, once the slots it overwrites
 // have been read.
 template <class L, int H>
-__device__ __forceinline__ void cg_pair_item(const float* __restrict__ in, float* __restrict__ out,
-                                             const CgMaps* __restrict__ maps, const Layout& lay, const PairK& k,
-                                             const Sched2& sc, int it, int zlo, int nzr, March& st, int* err,
-                                             long long budget) {
+__device__ __forceinline__ void cg_pair_item(const float* in, float* out, const CgMaps* __restrict__ maps,
+                                             const Layout& lay, const PairK& k, const Sched2& sc, int it, int zlo,
+                                             int nzr, March& st, int* err, long long budget) {
     using namespace pk;
     using C = CgTile<L, H>;
     using SH = Shells<L>;
@@ -681,7 +680,7 @@ __device__ __forceinline__ void cg_pair_end(const March& st, uint32_t bar) {
 
 template <class L, int H, int MINB>
 __global__ void __launch_bounds__(32 * (H + 1), MINB)
-    k_cg_pair(const float* __restrict__ in, float* __restrict__ out, const __grid_constant__ CgMaps maps, Layout lay,
+    k_cg_pair(const float* in, float* out, const __grid_constant__ CgMaps maps, Layout lay,
               PairK k, Sched2 sc, int zlo, int nzr, int* err, int* queue, long long budget) {
     using C = CgTile<L, H>;
     const uint32_t bar = cg_pair_begin<C>();

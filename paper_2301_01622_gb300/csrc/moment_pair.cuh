@@ -112,8 +112,7 @@ __device__ __forceinline__ void narrow(float2 v, S& lo, S& hi) {
 // without the copy in x alone): the copies that exist are the set bits of a
 // mask, so a node at one face runs one iteration.
 template <class S>
-__device__ __forceinline__ void store_ghosts(S* __restrict__ out, const Layout& lay, int x, int y, int z, const S* v,
-                                             bool y_only) {
+__device__ __forceinline__ void store_ghosts(S* out, const Layout& lay, int x, int y, int z, const S* v, bool y_only) {
     const unsigned xm = (x < kGhostX ? 1u : 0u) | (x >= lay.nx - kGhostX ? 2u : 0u);
     const unsigned ym = (y < lay.yo ? 1u : 0u) | (y >= lay.ny - lay.yo ? 2u : 0u);
     // copy k = 3 yk + xk: shift by 0, +n, -n in each direction
@@ -144,8 +143,7 @@ struct Step {
 
 template <class L, class S, int H, int MINB, class Op>
 __global__ void __launch_bounds__(32 * (H + 1), MINB)
-    k_moment_pair(const S* __restrict__ in, S* __restrict__ out, Layout lay, Op op, Sched sc, int zlo, int nzr, int ghosts,
-                  int* queue) {
+    k_moment_pair(const S* in, S* out, Layout lay, Op op, Sched sc, int zlo, int nzr, int ghosts, int* queue) {
     using namespace pk;
     using K = PairTile<L, H>;
     using SH = Shells<L>;
@@ -167,7 +165,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
     auto load = [&](S* v, size_t e) {
         if (LLB_IN(e + 9 * fs, 10 * lay.fs, kChkLoad)) {
 #pragma unroll
-            for (int f = 0; f < 10; ++f) v[f] = __ldg(in + e + f * fs);
+            for (int f = 0; f < 10; ++f) v[f] = load_dep(in + e + f * fs);
         }
     };
     const float2 zero = make_float2(0.0f, 0.0f);

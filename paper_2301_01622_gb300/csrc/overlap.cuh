@@ -10,6 +10,11 @@
 // visible.  dep_launch comes when a CTA has no item left: called at the start, the
 // waiting CTAs of the next step take the place of running ones (graph steps of 48^3
 // 6.4 us, so 5.6, without overlap 5.8; 32^3 5.0, 4.55, 4.75).  After a kernel that never calls dep_launch, or a copy, the launch is an ordinary one.
+//
+// What the kernel before wrote is read with load_dep and through pointers that are not
+// __restrict__.  The non-coherent load (__ldg, or what the compiler makes of a const
+// __restrict__ pointer) is for data that is read-only for the whole life of a kernel, and
+// the life of these begins while the kernel before still writes.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -20,6 +25,9 @@ namespace llb {
 
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class T>
+__device__ __forceinline__ T load_dep(const T* p) { return *p; }
 
 template <class... P, class... A>
 cudaError_t launch_overlapped(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t stream, A&&... args) {
