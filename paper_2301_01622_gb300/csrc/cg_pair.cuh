@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "cg_kernel.cuh"
+#include "cg_stages.cuh"
 #include "overlap.cuh"
 #include "pair_march.cuh"
 #include "tma.cuh"
@@ -303,7 +304,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
     auto m_slot = [&](unsigned n) { return reinterpret_cast<const float*>(base + C::M_OFF + (n & 1) * C::M_SLOT); };
     // load the group of step s (one thread)
     auto stage = [&](int s, unsigned n) {
-        const uint32_t b = bar + 8 * (n & 1);
+        const uint32_t b = bar + 8 * Stages::bar(n);
         const bool mom = s >= za - 1, rd = s < zb;
         mbar_arrive_expect_tx(b, (mom ? C::M_BYTES : 0) + (rd ? C::R_BYTES : 0));
         if (rd)
@@ -313,11 +314,17 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
             tma_load_4d(smem_u32(base + C::M_OFF + (n & 1) * C::M_SLOT), &maps->m, x0 - 4 + lay.xo, y0 - 1 + lay.yo,
                         pmod2(s, nz), 2, b);
     };
-    auto await = [&]() {
-        if (!st.dead && !mbar_wait_bounded(bar + 8 * (st.n & 1), (st.n >> 1) & 1, budget)) {
-            atomicExch(err, 3);
-            st.dead = true;
-        }
+    // Wait for the group of step s.  After a wait that gave up, the thread that issues the
+    // copies lets those in flight land (bounded) before it goes on: later the barriers'
+    // phases no longer tell which they were, and a CTA must not end with copies on the way
+    // into its shared memory.
+    auto await = [&](int s) {
+        if (st.dead || mbar_wait_bounded(bar + 8 * Stages::bar(st.n), Stages::parity(st.n), budget)) return;
+        atomicExch(err, 3);
+        st.dead = true;
+        if (w == H && lane == 0)
+            for (unsigned q = st.n; q != Stages::in_flight_end(st.n, s, zb); ++q)
+                mbar_wait_bounded(bar + 8 * Stages::bar(q), Stages::parity(q), kDrainBudget);
     };
 
     // The march of every warp: source planes s = za - 4 .. zb; the first three only
@@ -337,7 +344,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
 #pragma unroll 1
         for (int s = za - 4;; ++s) {
             __syncwarp();
-            await();
+            await(s);
             float2 gx, gy, gz;
             const float* const P = f2(PH + pb * PN);
             gr.advance([&](int dy, int dx) {
@@ -423,7 +430,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
 
 #pragma unroll 1
     for (int s = za - 4;; ++s) {
-        await();
+        await(s);
         float2 gx, gy, gz;
         {
             const float2* const Pp = PH + pb * PN + p1 - lane;
@@ -658,7 +665,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
 
 // Staging barriers up; every warp of the CTA.
 template <class C>
-__device__ __forceinline__ uint32_t cg_pair_begin() {
+__device__ __forceinline__ void cg_pair_begin() {
     extern __shared__ unsigned char smem_raw[];
     const uint32_t base = smem_u32(smem_raw), bar = base + ((128 - (base & 127)) & 127) + C::BAR_OFF;
     if (threadIdx.x == 0) {
@@ -667,15 +674,6 @@ __device__ __forceinline__ uint32_t cg_pair_begin() {
         fence_barrier_init();
     }
     __syncthreads();
-    return bar;
-}
-
-// Results out; after a wait that gave up, the copies still in flight in (bounded).
-template <class C>
-__device__ __forceinline__ void cg_pair_end(const March& st, uint32_t bar) {
-    if (threadIdx.x == 0) bulk_wait();
-    if (st.dead && threadIdx.x == C::NT - 32)
-        for (int b = 0; b < 2; ++b) mbar_wait_bounded(bar + 8 * ((st.n + b) & 1), ((st.n + b) >> 1) & 1, 100000000LL);
 }
 
 template <class L, int H, int MINB>
@@ -683,7 +681,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
     k_cg_pair(const float* in, float* out, const __grid_constant__ CgMaps maps, Layout lay,
               PairK k, Sched2 sc, int zlo, int nzr, int* err, int* queue, long long budget) {
     using C = CgTile<L, H>;
-    const uint32_t bar = cg_pair_begin<C>();
+    cg_pair_begin<C>();
     March st;
     // Items from a queue (queue[0]: next item, queue[1]: CTAs done): those that hold an
     // interface take longer.  The last CTA to leave resets it for the next launch.
@@ -698,7 +696,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         cg_pair_item<L, H>(in, out, &maps, lay, k, sc, it, zlo, nzr, st, err, budget);
     }
     dep_launch();
-    cg_pair_end<C>(st, bar);
+    if (threadIdx.x == 0) bulk_wait();  // results out
     if (threadIdx.x == 0 && atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {
         queue[0] = 0;
         queue[1] = 0;
@@ -712,7 +710,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
                     int* __restrict__ next, long long budget) {
     using C = CgTile<L, H>;
     __shared__ int s_it;
-    const uint32_t bar = cg_pair_begin<C>();
+    cg_pair_begin<C>();
     March st;
     for (;;) {
         if (threadIdx.x == 0) s_it = atomicAdd(next, 1);
@@ -737,7 +735,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         cg_pair_item<L, H>(static_cast<const float*>(d.in), static_cast<float*>(d.out), maps + lo, d.lay, k, sc,
                            it - d.item_begin, 0, d.lay.nz, st, d.err, budget);
     }
-    cg_pair_end<C>(st, bar);
+    if (threadIdx.x == 0) bulk_wait();  // results out
 }
 
 // Tiles of 28 x 10, two CTAs of six warps per SM (168 registers, no spills; 113 KB

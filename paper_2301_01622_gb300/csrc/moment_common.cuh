@@ -24,10 +24,6 @@
 namespace llb {
 namespace mom {
 
-// cycles (~50 ms) to let this CTA's copies in flight land after an abort: a
-// 16 KB box arrives within microseconds even under heavy load
-constexpr long long kDrainBudget = 100000000LL;
-
 // Ten shifted moments of node idx from a state of element type S (converted to T).
 // Ten shifted moments of node idx (index of the node in the state buffer p).
 template <class T, class S>

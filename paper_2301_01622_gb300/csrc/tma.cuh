@@ -58,6 +58,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     return true;
 }
 
+// cycles (~50 ms) to let this CTA's copies in flight land after an abort: a
+// 16 KB box arrives within microseconds even under heavy load
+constexpr long long kDrainBudget = 100000000LL;
+
 // 4D tiled TMA load of one box into shared memory, completion signalled on `bar`.
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                             uint32_t bar) {
