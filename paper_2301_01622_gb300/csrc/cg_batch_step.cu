@@ -43,7 +43,7 @@ cudaError_t cg_batch_run_v(const llb_ctx& c, const BatchDom* doms, const CgMaps*
     if constexpr (V::PAIR) {
         using K = CgTile<L, kPairH>;
         k_cg_pair_batch<L, kPairH, kPairCtas><<<grid, K::NT, K::smem_bytes, c.stream>>>(
-            doms, maps, ndom, total, pair_constants<L>(c), next, wait_cycles(c));
+            doms, maps, ndom, total, pair_constants<L>(c), next, wait_bounds(c));
     } else {
         using C = CGCfg<L, T, V::BX, V::BY>;
         k_cg_batch<L, T, V::BX, V::BY, V::MINB, V::FAST, V::ROLLED><<<grid, C::NT, C::smem_bytes, c.stream>>>(

@@ -250,6 +250,13 @@ static __device__ __noinline__ int near_contact(const float* r1, const float* dd
     return got;
 }
 
+// Bound of a wait in cycles, and bytes that a barrier is armed for beyond those its copies
+// deliver (fault injection: 0 in normal use).
+struct WaitK {
+    long long budget;
+    int extra_tx;
+};
+
 // State that a CTA carries from item to item.
 struct March {
     int par = 0;       // plane parity of the doubled exchange rows
@@ -266,7 +273,7 @@ struct March {
 template <class L, int H>
 __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const CgMaps* __restrict__ maps,
                                              const Layout& lay, const PairK& k, const Sched2& sc, int it, int zlo,
-                                             int nzr, March& st, int* err, long long budget) {
+                                             int nzr, March& st, int* err, const WaitK& wk) {
     using namespace pk;
     using C = CgTile<L, H>;
     using SH = Shells<L>;
@@ -306,7 +313,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
     auto stage = [&](int s, unsigned n) {
         const uint32_t b = bar + 8 * Stages::bar(n);
         const bool mom = s >= za - 1, rd = s < zb;
-        mbar_arrive_expect_tx(b, (mom ? C::M_BYTES : 0) + (rd ? C::R_BYTES : 0));
+        mbar_arrive_expect_tx(b, (mom ? C::M_BYTES : 0) + (rd ? C::R_BYTES : 0) + wk.extra_tx);
         if (rd)
             tma_load_4d(smem_u32(base + C::R_OFF + (n & 3) * C::R_SLOT), &maps->rd, x0 - 4 + lay.xo, y0 - 2 + lay.yo,
                         pmod2(s + 2, nz), 0, b);
@@ -319,7 +326,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
     // phases no longer tell which they were, and a CTA must not end with copies on the way
     // into its shared memory.
     auto await = [&](int s) {
-        if (st.dead || mbar_wait_bounded(bar + 8 * Stages::bar(st.n), Stages::parity(st.n), budget)) return;
+        if (st.dead || mbar_wait_bounded(bar + 8 * Stages::bar(st.n), Stages::parity(st.n), wk.budget)) return;
         atomicExch(err, 3);
         st.dead = true;
         if (w == H && lane == 0)
@@ -679,7 +686,7 @@ __device__ __forceinline__ void cg_pair_begin() {
 template <class L, int H, int MINB>
 __global__ void __launch_bounds__(32 * (H + 1), MINB)
     k_cg_pair(const float* in, float* out, const __grid_constant__ CgMaps maps, Layout lay,
-              PairK k, Sched2 sc, int zlo, int nzr, int* err, int* queue, long long budget) {
+              PairK k, Sched2 sc, int zlo, int nzr, int* err, int* queue, WaitK wk) {
     using C = CgTile<L, H>;
     cg_pair_begin<C>();
     March st;
@@ -693,7 +700,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         const int it = s_it;
         __syncthreads();
         if (it >= sc.nitems) break;
-        cg_pair_item<L, H>(in, out, &maps, lay, k, sc, it, zlo, nzr, st, err, budget);
+        cg_pair_item<L, H>(in, out, &maps, lay, k, sc, it, zlo, nzr, st, err, wk);
     }
     dep_launch();
     if (threadIdx.x == 0) bulk_wait();  // results out
@@ -707,7 +714,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
 template <class L, int H, int MINB>
 __global__ void __launch_bounds__(32 * (H + 1), MINB)
     k_cg_pair_batch(const BatchDom* __restrict__ doms, const CgMaps* __restrict__ maps, int ndom, int total, PairK k,
-                    int* __restrict__ next, long long budget) {
+                    int* __restrict__ next, WaitK wk) {
     using C = CgTile<L, H>;
     __shared__ int s_it;
     cg_pair_begin<C>();
@@ -733,7 +740,7 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
         }
         if (threadIdx.x == 0) acquire_tensormap(&maps[lo].out);
         cg_pair_item<L, H>(static_cast<const float*>(d.in), static_cast<float*>(d.out), maps + lo, d.lay, k, sc,
-                           it - d.item_begin, 0, d.lay.nz, st, d.err, budget);
+                           it - d.item_begin, 0, d.lay.nz, st, d.err, wk);
     }
     if (threadIdx.x == 0) bulk_wait();  // results out
 }
@@ -758,7 +765,10 @@ inline bool cg_pair_maps(const llb_ctx& c, const void* in, void* out, CgMaps* m)
            encode_f32_map(static_cast<float*>(out) + y.at(0, 0, 0), inner, strides, res, &m->out);
 }
 
-inline long long wait_cycles(const llb_ctx& c) { return (long long)c.params.wait_budget_ms * 2000000LL; }
+// device clock ~2 GHz: cycles per millisecond
+inline WaitK wait_bounds(const llb_ctx& c) {
+    return {(long long)c.params.wait_budget_ms * 2000000LL, (c.params.debug_flags & 1) ? 1 : 0};
+}
 
 // Chunk length of a box whose items go through the queue on `grid` CTAs.  A step
 // of an item costs about its planes plus 3.5 to fill the pipeline.  Without near

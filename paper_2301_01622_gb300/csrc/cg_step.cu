@@ -39,7 +39,7 @@ cudaError_t cg_run_v(const llb_ctx& c, const void* in, void* out, int zlo, int z
         return launch_overlapped(k_cg_pair<L, kPairH, kPairCtas>, grid, K::NT, K::smem_bytes, st,
                                  static_cast<const float*>(in), static_cast<float*>(out), maps, c.lay,
                                  pair_constants<L>(c), sc, zlo, zhi - zlo, static_cast<int*>(c.err_dev),
-                                 static_cast<int*>(c.queue_dev), wait_cycles(c));
+                                 static_cast<int*>(c.queue_dev), wait_bounds(c));
     } else {
         using C = CGCfg<L, T, V::BX, V::BY>;
         const Sched2 sc = plan2(c.nx, c.ny, zhi - zlo, V::BX, V::BY, grid);

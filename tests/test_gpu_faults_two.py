@@ -1,0 +1,66 @@
+"""A device wait of the two-component step that cannot complete (its barrier is armed for
+a byte that never arrives; the copies themselves land) runs out after its bound, is
+reported as LLB_ETIMEOUT by the calls that synchronise and leaves the CUDA context usable."""
+import numpy as np
+import pytest
+
+from oracle import D3Q19, lb
+from oracle import two_component as tc
+from paper_2301_01622_gb300 import inputs, llb
+
+pytestmark = pytest.mark.gpu
+
+SHAPE = (64, 40, 24)
+STUCK = dict(ncomp=2, storage=llb.LLB_F32, wait_budget_ms=20, debug_flags=1)
+
+
+def _drop(shape):
+    nx, ny, nz = shape
+    r1, r2, u = inputs.droplets(nx, ny, nz, [(nx / 2, ny / 2, nz / 2)], [min(shape) / 4], [(0.02, 0, 0)])
+    return np.concatenate([r1[None], r2[None], lb.equilibrium_moments(r1 + r2, u)[1:]])
+
+
+def _status(fn, *args):
+    with pytest.raises(llb.LLBError) as e:
+        fn(*args)
+    return e.value.status
+
+
+def _device_still_works():
+    shape = (20, 12, 8)
+    m0 = _drop(shape)
+    ctx = llb.llb_create(*shape, 19, 0.9, llb.llb_params_default(storage=llb.LLB_F32, ncomp=2))
+    try:
+        llb.llb_init_moments(ctx, m0)
+        llb.llb_step(ctx, 2)
+        got = llb.llb_get_moments(ctx, np.empty_like(m0))
+    finally:
+        llb.llb_destroy(ctx)
+    ref = tc.run_moment_only(m0, D3Q19, 0.9, tc.CGParams(g_min=1e-6), 2)
+    assert np.abs(got - ref).max() < 1e-5
+
+
+@pytest.mark.parametrize("q", [19, 27])
+@pytest.mark.parametrize("graph", [False, True], ids=["step", "graph"])
+def test_single_box_reports_the_timeout(q, graph):
+    m0 = _drop(SHAPE)
+    for read in (llb.llb_synchronize, lambda c: llb.llb_get_moments(c, np.empty_like(m0)), llb.llb_diagnostics):
+        ctx = llb.llb_create(*SHAPE, q, 0.9, llb.llb_params_default(**STUCK))
+        try:
+            llb.llb_init_moments(ctx, m0)
+            (llb.llb_step_graph if graph else llb.llb_step)(ctx, 2)
+            assert _status(read, ctx) == llb.LLB_ETIMEOUT
+            assert _status(llb.llb_step, ctx, 1) == llb.LLB_ESTATE  # sticky from now on
+        finally:
+            llb.llb_destroy(ctx)
+    _device_still_works()
+
+
+def test_host_step_reports_the_timeout():
+    m0 = _drop(SHAPE)
+    ctx = llb.llb_create(*SHAPE, 19, 0.9, llb.llb_params_default(**STUCK))
+    try:
+        assert _status(llb.llb_step_host, ctx, m0, np.empty_like(m0), 2) == llb.LLB_ETIMEOUT
+    finally:
+        llb.llb_destroy(ctx)
+    _device_still_works()
