@@ -321,6 +321,10 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
             tma_load_4d(smem_u32(base + C::M_OFF + (n & 1) * C::M_SLOT), &maps->m, x0 - 4 + lay.xo, y0 - 1 + lay.yo,
                         pmod2(s, nz), 2, b);
     };
+    // Items taken after a wait gave up are not computed from loaded data: their box reports
+    // it too, whichever box the wait was for.
+    if (st.dead) atomicExch(err, 3);
+
     // Wait for the group of step s.  After a wait that gave up, the thread that issues the
     // copies lets those in flight land (bounded) before it goes on: later the barriers'
     // phases no longer tell which they were, and a CTA must not end with copies on the way

@@ -64,3 +64,21 @@ def test_host_step_reports_the_timeout():
     finally:
         llb.llb_destroy(ctx)
     _device_still_works()
+
+
+@pytest.mark.parametrize("graph", [False, True], ids=["step", "graph"])
+def test_every_box_of_a_batch_reports_the_timeout(graph):
+    """More boxes than CTAs: a CTA whose wait has given up goes on to items of other boxes,
+    and each of those has to report that its step was not done."""
+    dims = [(8, 6, 5)] * 700  # one item each; at most four CTAs on each of up to 160 SMs
+    b = llb.llb_batch_create(dims, 19, 0.9, llb.llb_params_default(**STUCK))
+    try:
+        m0 = _drop(dims[0])
+        for k in range(len(dims)):
+            llb.llb_init_moments(llb.llb_batch_domain(b, k), m0)
+        (llb.llb_batch_step_graph if graph else llb.llb_batch_step)(b, 1)
+        got = [_status(llb.llb_synchronize, llb.llb_batch_domain(b, k)) for k in range(len(dims))]
+        assert got == [llb.LLB_ETIMEOUT] * len(dims)
+    finally:
+        llb.llb_batch_destroy(b)
+    _device_still_works()
