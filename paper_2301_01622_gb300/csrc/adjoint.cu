@@ -1180,6 +1180,9 @@ extern "C" int llb_adjoint_in(llb_ctx* c, int nsteps, int every, const void* dev
     }
     double domega = 0.0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&domega, acc, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    // the error word of the forward steps: this call synchronises, so it reports a wait that gave up
+    int gave_up = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&gave_up, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     // restore the initial state
     if (e == cudaSuccess && nseg > 0 && !direct)
         e = cudaMemcpyAsync(c->buf[cur0], ck, c->state_bytes, cudaMemcpyDeviceToDevice, c->stream);
@@ -1191,6 +1194,11 @@ extern "C" int llb_adjoint_in(llb_ctx* c, int nsteps, int every, const void* dev
         c->sticky = LLB_ECUDA;
         c->msg = std::string("adjoint: ") + cudaGetErrorString(e);
         return LLB_ECUDA;
+    }
+    if (gave_up) {
+        c->sticky = LLB_ETIMEOUT;
+        c->msg = "adjoint: a device wait gave up (a TMA load or a plane barrier did not complete)";
+        return LLB_ETIMEOUT;
     }
     // omega = 1 / tau
     if (dtau) *dtau = -domega / (c->tau * c->tau);

@@ -82,3 +82,23 @@ def test_every_box_of_a_batch_reports_the_timeout(graph):
     finally:
         llb.llb_batch_destroy(b)
     _device_still_works()
+
+
+@pytest.mark.parametrize("params", [dict(STUCK, grad_eps=0.05), dict(storage=llb.LLB_F32, kernel=llb.LLB_KERNEL_TMA,
+                                    wait_budget_ms=20, debug_flags=1)], ids=["two-component", "one-component-tma"])
+def test_adjoint_reports_the_timeout(params):
+    """The forward steps of a gradient wait too, and the call synchronises."""
+    import torch
+
+    m0 = _drop(SHAPE)
+    if params.get("ncomp", 1) == 1:
+        m0 = np.concatenate([m0[:1] + m0[1:2], m0[2:]])
+    g = torch.ones(m0.shape, dtype=torch.float32, device="cuda")
+    ctx = llb.llb_create(*SHAPE, 19, 0.9, llb.llb_params_default(**params))
+    try:
+        llb.llb_init_moments(ctx, m0)
+        assert _status(llb.llb_adjoint, ctx, 4, g, torch.empty_like(g)) == llb.LLB_ETIMEOUT
+        assert _status(llb.llb_step, ctx, 1) == llb.LLB_ESTATE
+    finally:
+        llb.llb_destroy(ctx)
+    _device_still_works()
