@@ -41,7 +41,9 @@ cudaError_t launch_overlapped(void (*kern)(P...), int grid, int block, size_t sm
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here: the next launch must not find it again
+    return e;
 }
 
 }  // namespace llb
