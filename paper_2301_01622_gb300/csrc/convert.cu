@@ -73,46 +73,84 @@ __device__ __forceinline__ void put(T* __restrict__ st, const Layout& L, int x, 
 template <class C, class T>
 constexpr bool kTwoFloat = std::is_same<C, float>::value && !std::is_same<T, double>::value;
 
-// Total density rho = v[0] (+ v[1]) as rounded value and remainder.
-template <int NC, class V>
-__device__ __forceinline__ void total(const V* v, V& h, V& l) {
-    h = v[0];
-    l = V(0);
-    if constexpr (NC == 2) {
-        if constexpr (std::is_same<V, float>::value) {
-            const Two s = Two::sum(v[0], v[1]);
-            h = s.h;
-            l = s.l;
-        } else {
-            h = v[0] + v[1];
-        }
-    }
+// Whether pairs of floats hold the arithmetic of a node: its total density h and what is
+// combined with it finite and far from both ends of the range.  An infinity or NaN has no
+// low part, and very small values lose it; such nodes take the FP64 form.
+__device__ __forceinline__ bool pairs_hold(float h, float a, float b, float c) {
+    return h >= 0x1p-60f && h <= 0x1p60f && fabsf(a) <= 0x1p60f && fabsf(b) <= 0x1p60f && fabsf(c) <= 0x1p60f;
 }
 
-__device__ __forceinline__ double less_one(double h, double) { return h - 1.0; }
-__device__ __forceinline__ float less_one(float h, float l) {
-    const Two s = Two::sum(h, -1.0f);
-    return __fadd_rn(s.h, __fadd_rn(s.l, l));
-}
 // P - rho / 3
-__device__ __forceinline__ double less_third(double p, double h, double) { return p - kCs2 * h; }
-__device__ __forceinline__ float less_third(float p, float h, float l) {
-    const Two t = third(h, l), s = Two::sum(p, -t.h);
+__device__ __forceinline__ float less_third(float p, const Two& rho) {
+    const Two t = third(rho.h, rho.l), s = Two::sum(p, -t.h);
     return __fadd_rn(s.h, __fsub_rn(s.l, t.l));
 }
-// A + (1 + d) / 3
-__device__ __forceinline__ double plus_third(double a, double d) { return a + kCs2 * (1.0 + d); }
-__device__ __forceinline__ float plus_third(float a, float d) {
-    const Two r = Two::sum(1.0f, d), t = third(r.h, r.l), s = Two::sum(a, t.h);
+// A + rho / 3
+__device__ __forceinline__ float plus_third(float a, const Two& rho) {
+    const Two t = third(rho.h, rho.l), s = Two::sum(a, t.h);
     return __fadd_rn(s.h, __fadd_rn(s.l, t.l));
 }
-__device__ __forceinline__ double one_plus(double d) { return 1.0 + d; }
-__device__ __forceinline__ float one_plus(float d) { return __fadd_rn(1.0f, d); }
-// 1 + d - r1
-__device__ __forceinline__ double other_colour(double d, double r1) { return (1.0 + d) - r1; }
-__device__ __forceinline__ float other_colour(float d, float r1) {
-    const Two r = Two::sum(1.0f, d), s = Two::sum(r.h, -r1);
-    return __fadd_rn(s.h, __fadd_rn(s.l, r.l));
+
+// State (rho1,) d, j, A of canonical (rho or rho1, rho2), j, P; returns whether the total
+// density is not positive or, in FP64, not finite.
+template <int NC>
+__device__ __forceinline__ bool to_state(const double* v, double* o) {
+    const double rho = NC == 2 ? v[0] + v[1] : v[0];
+    if constexpr (NC == 2) o[0] = v[0];
+    o[NC - 1] = rho - 1.0;
+#pragma unroll
+    for (int f = NC; f < 9 + NC; ++f) o[f] = f < NC + 3 || f >= NC + 6 ? v[f] : v[f] - kCs2 * rho;
+    return bad_rho(rho);
+}
+template <int NC>
+__device__ __forceinline__ bool to_state(const float* v, float* o) {
+    Two rho{v[0], 0.0f};
+    if constexpr (NC == 2) rho = Two::sum(v[0], v[1]);
+    if (!pairs_hold(rho.h, v[NC + 3], v[NC + 4], v[NC + 5])) {
+        double w[9 + NC], r[9 + NC];
+#pragma unroll
+        for (int f = 0; f < 9 + NC; ++f) w[f] = (double)v[f];
+        const bool bad = to_state<NC>(w, r);
+#pragma unroll
+        for (int f = 0; f < 9 + NC; ++f) o[f] = (float)r[f];
+        return bad;
+    }
+    if constexpr (NC == 2) o[0] = v[0];
+    const Two d = Two::sum(rho.h, -1.0f);
+    o[NC - 1] = __fadd_rn(d.h, __fadd_rn(d.l, rho.l));
+#pragma unroll
+    for (int f = NC; f < 9 + NC; ++f) o[f] = f < NC + 3 || f >= NC + 6 ? v[f] : less_third(v[f], rho);
+    return false;
+}
+
+// The way back.
+template <int NC>
+__device__ __forceinline__ void to_canon(const double* v, double* o) {
+    const double rho = 1.0 + v[NC - 1];
+    o[0] = NC == 2 ? v[0] : rho;
+    if constexpr (NC == 2) o[1] = rho - v[0];
+#pragma unroll
+    for (int f = NC; f < 9 + NC; ++f) o[f] = f < NC + 3 || f >= NC + 6 ? v[f] : v[f] + kCs2 * rho;
+}
+template <int NC>
+__device__ __forceinline__ void to_canon(const float* v, float* o) {
+    const Two rho = Two::sum(1.0f, v[NC - 1]);
+    if (!pairs_hold(rho.h, v[NC + 3], v[NC + 4], v[NC + 5]) || (NC == 2 && !(fabsf(v[0]) <= 0x1p60f))) {
+        double w[9 + NC], r[9 + NC];
+#pragma unroll
+        for (int f = 0; f < 9 + NC; ++f) w[f] = (double)v[f];
+        to_canon<NC>(w, r);
+#pragma unroll
+        for (int f = 0; f < 9 + NC; ++f) o[f] = (float)r[f];
+        return;
+    }
+    o[0] = NC == 2 ? v[0] : rho.h;
+    if constexpr (NC == 2) {
+        const Two s = Two::sum(rho.h, -v[0]);
+        o[1] = __fadd_rn(s.h, __fadd_rn(s.l, rho.l));
+    }
+#pragma unroll
+    for (int f = NC; f < 9 + NC; ++f) o[f] = f < NC + 3 || f >= NC + 6 ? v[f] : plus_third(v[f], rho);
 }
 
 // Nodes i0 .. i1-1 of the dense canonical order (whole planes for a z-range).
@@ -124,24 +162,15 @@ __global__ void __launch_bounds__(256) k_canon_to_shifted(const C* __restrict__ 
     constexpr int NF = 9 + NC;
     const size_t N = (size_t)L.nx * L.ny * L.nz;
     for (size_t i = i0 + blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
-        V v[NF], o[NF], h, l;
+        V v[NF], o[NF];
 #pragma unroll
         for (int f = 0; f < NF; ++f) v[f] = (V)__ldg(canon + f * N + i);
-        total<NC>(v, h, l);
         // the total density must be positive; a colour density may dip slightly
         // below zero (the stepped colour-gradient field does so near interfaces)
-        bool b = !(h > V(0)) || (std::is_same<V, double>::value && !isfinite(h));
+        bool b = to_state<NC>(v, o);
 #pragma unroll
         for (int f = 0; f < NF; ++f) b = b || !isfinite(v[f]);
         if (b && bad) atomicOr(bad, 1);
-        if constexpr (NC == 2) o[0] = v[0];
-        o[NC - 1] = less_one(h, l);
-#pragma unroll
-        for (int f = NC; f < NC + 3; ++f) o[f] = v[f];
-#pragma unroll
-        for (int f = NC + 3; f < NC + 6; ++f) o[f] = less_third(v[f], h, l);
-#pragma unroll
-        for (int f = NC + 6; f < NF; ++f) o[f] = v[f];
         int x, y, z;
         decode(L, i, x, y, z);
         put<T, NF>(st, L, x, y, z, o);
@@ -165,19 +194,10 @@ __global__ void __launch_bounds__(256) k_shifted_to_canon(const T* __restrict__ 
             if constexpr (IsNarrow<T>::value) v[f] = cv_field<V>(t, f);
             else v[f] = (V)t;
         }
-        const V d = v[NC - 1];
-        if constexpr (NC == 2) {
-            canon[i] = (C)v[0];
-            canon[N + i] = (C)other_colour(d, v[0]);
-        } else {
-            canon[i] = (C)one_plus(d);
-        }
+        V o[NF];
+        to_canon<NC>(v, o);
 #pragma unroll
-        for (int f = NC; f < NC + 3; ++f) canon[f * N + i] = (C)v[f];
-#pragma unroll
-        for (int f = NC + 3; f < NC + 6; ++f) canon[f * N + i] = (C)plus_third(v[f], d);
-#pragma unroll
-        for (int f = NC + 6; f < NF; ++f) canon[f * N + i] = (C)v[f];
+        for (int f = 0; f < NF; ++f) canon[f * N + i] = (C)o[f];
     }
 }
 
