@@ -4,8 +4,9 @@
 // canonical (one component): rho, j_x, j_y, j_z, P_xx, P_yy, P_zz, P_xy, P_xz, P_yz
 // shifted storage:           d = rho - 1, j, A = P - cs^2 rho I
 // Equilibrium (second moment of Eq. (5)): P^eq = cs^2 rho I + rho u u, so
-// A^eq = rho u u.  All conversions round once: they compute in FP64, or in pairs
-// of floats where both sides are at most FP32.
+// A^eq = rho u u.  All conversions compute in FP64, or in several floats where both
+// sides are at most FP32, and round the result to FP32 or FP64 once (16-bit states
+// round that once more, to their format).
 // Two components: canonical rho1, rho2, j, P; state rho1, d = rho1 + rho2 - 1,
 // j, A (rho1 needs no shift: it lies in [0, rho]).
 // Canonical buffers are dense; the shifted state follows the context's
@@ -67,28 +68,30 @@ __device__ __forceinline__ void put(T* __restrict__ st, const Layout& L, int x, 
 }
 
 // The maps between canonical and stored values, rounded once.  From FP32 to a
-// state of at most FP32 they run on pairs of floats: in FP64 the two conversions
+// state of at most FP32 they run on sums of floats (twofloat.cuh): in FP64 the two conversions
 // of every value and the arithmetic kept the FP64 pipe 80 % busy and took three
 // times as long as the memory needs.
 template <class C, class T>
 constexpr bool kTwoFloat = std::is_same<C, float>::value && !std::is_same<T, double>::value;
 
-// Whether pairs of floats hold the arithmetic of a node: its total density h and what is
+// Whether sums of floats hold the arithmetic of a node: its total density h and what is
 // combined with it finite and far from both ends of the range.  An infinity or NaN has no
 // low part, and very small values lose it; such nodes take the FP64 form.
 __device__ __forceinline__ bool pairs_hold(float h, float a, float b, float c) {
     return h >= 0x1p-60f && h <= 0x1p60f && fabsf(a) <= 0x1p60f && fabsf(b) <= 0x1p60f && fabsf(c) <= 0x1p60f;
 }
 
-// P - rho / 3
+// P - rho / 3 and A + rho / 3 of a density rho = h + l, rounded once.  (In FP64 the product
+// with 1/3 is rounded to 2^-54 of rho first; where P is close to rho / 3 that shows in A.)
 __device__ __forceinline__ float less_third(float p, const Two& rho) {
-    const Two t = third(rho.h, rho.l), s = Two::sum(p, -t.h);
-    return __fadd_rn(s.h, __fsub_rn(s.l, t.l));
+    const Third t(rho.h, rho.l);
+    const Two s = Two::sum(p, -t.a), x = Two::sum(s.l, -t.b);
+    return round_sum(s.h, x.h, __fsub_rn(x.l, t.c));
 }
-// A + rho / 3
 __device__ __forceinline__ float plus_third(float a, const Two& rho) {
-    const Two t = third(rho.h, rho.l), s = Two::sum(a, t.h);
-    return __fadd_rn(s.h, __fadd_rn(s.l, t.l));
+    const Third t(rho.h, rho.l);
+    const Two s = Two::sum(a, t.a), x = Two::sum(s.l, t.b);
+    return round_sum(s.h, x.h, __fadd_rn(x.l, t.c));
 }
 
 // State (rho1,) d, j, A of canonical (rho or rho1, rho2), j, P; returns whether the total
@@ -116,8 +119,7 @@ __device__ __forceinline__ bool to_state(const float* v, float* o) {
         return bad;
     }
     if constexpr (NC == 2) o[0] = v[0];
-    const Two d = Two::sum(rho.h, -1.0f);
-    o[NC - 1] = __fadd_rn(d.h, __fadd_rn(d.l, rho.l));
+    o[NC - 1] = NC == 2 ? round_sum(-1.0f, v[0], v[NC - 1]) : __fsub_rn(v[0], 1.0f);
 #pragma unroll
     for (int f = NC; f < 9 + NC; ++f) o[f] = f < NC + 3 || f >= NC + 6 ? v[f] : less_third(v[f], rho);
     return false;
@@ -145,10 +147,7 @@ __device__ __forceinline__ void to_canon(const float* v, float* o) {
         return;
     }
     o[0] = NC == 2 ? v[0] : rho.h;
-    if constexpr (NC == 2) {
-        const Two s = Two::sum(rho.h, -v[0]);
-        o[1] = __fadd_rn(s.h, __fadd_rn(s.l, rho.l));
-    }
+    if constexpr (NC == 2) o[1] = round_sum(1.0f, v[1], -v[0]);
 #pragma unroll
     for (int f = NC; f < 9 + NC; ++f) o[f] = f < NC + 3 || f >= NC + 6 ? v[f] : plus_third(v[f], rho);
 }

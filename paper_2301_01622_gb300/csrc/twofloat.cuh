@@ -36,12 +36,27 @@ struct Two {
     }
 };
 
-// (h + l) / 3
-__device__ __forceinline__ Two third(float h, float l) {
-    constexpr float c = (float)(1.0 / 3.0), ce = (float)(1.0 / 3.0 - (double)c);
-    Two p = Two::prod(h, c);
-    p.l = __fmaf_rn(l, c, __fmaf_rn(h, ce, p.l));
-    return p;
+// a + b + c rounded once: b + c and a + (b + c) as exact pairs, their low parts added with
+// rounding to odd, which keeps the last addition from rounding a second time (Boldo and
+// Melquiond, "Emulation of a FMA and correctly rounded sums", 2008).
+__device__ __forceinline__ float round_sum(float a, float b, float c) {
+    const Two u = Two::sum(b, c), t = Two::sum(a, u.h), v = Two::sum(t.l, u.l);
+    float odd = v.h;
+    if (v.l != 0.0f && !(__float_as_uint(odd) & 1u))  // inexact and even: the neighbour on the side of the rest
+        odd = __uint_as_float(__float_as_uint(odd) + ((v.l > 0.0f) == (odd > 0.0f) ? 1u : ~0u));
+    return __fadd_rn(t.h, odd);
 }
+
+// (h + l) / 3 as three floats: quotients of the remainders, which are exact.  Error about 2^-70.
+struct Third {
+    float a, b, c;
+    __device__ __forceinline__ Third(float h, float l) {
+        constexpr float q = (float)(1.0 / 3.0);
+        a = __fmul_rn(h, q);
+        const Two r = Two::sum(__fmaf_rn(-3.0f, a, h), l);
+        b = __fmul_rn(r.h, q);
+        c = __fmul_rn(__fadd_rn(__fmaf_rn(-3.0f, b, r.h), r.l), q);
+    }
+};
 
 }  // namespace llb
