@@ -6,8 +6,9 @@
 // reduces in registers, then warp shuffles, then across the block's warps
 // through shared memory, and writes one row of partials per block to a
 // scratch array.  Pass 2: one block reduces the rows in a fixed order.  The
-// result is deterministic for a given grid.  The sums are FP64 for FP64 states
-// and carry at least its 46 leading bits for the others.
+// result is deterministic for a given grid.  The sums of a thread and a warp are
+// FP64 for FP64 data; for FP32 and 16-bit data they are sums of three floats,
+// which are at least as accurate, and FP64 where those overflow.
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -49,8 +50,8 @@ __device__ __forceinline__ Part warp_reduce(Part p) {
     return p;
 }
 
-// Sums of one thread.  States and inputs of at most FP32 are summed as pairs of
-// floats (twofloat.cuh): the FP64 form kept the FP64 pipe 79 % busy and took 106 us
+// Sums of one thread.  States and inputs of at most FP32 are summed in three floats
+// (Sum3, twofloat.cuh): the FP64 form kept the FP64 pipe 79 % busy and took 106 us
 // for the 92 MB of a 128^3 two-component state.
 template <bool WIDE>
 struct Sums;
@@ -89,17 +90,17 @@ struct Sums<true> {  // FP64 values
         v[6] = fmin(v[6], rho);
         if (!finite) v[7] = 1.0;
     }
-    __device__ __forceinline__ Part row() const {
-        Part p;
+    __device__ __forceinline__ bool row(Part& p) const {
         for (int k = 0; k < kRow; ++k) p.v[k] = v[k];
-        return warp_reduce(p);
+        p = warp_reduce(p);
+        return true;
     }
 };
 
 template <>
 struct Sums<false> {  // FP32 values
-    Two d, jx, jy, jz, in, all;  // in: sum of the droplet density (one component: of d) where it exceeds 0.5
-    float dmin = FLT_MAX, rmin = FLT_MAX;
+    Sum3 d, jx, jy, jz, in, all;  // in: sum of the droplet density (one component: of d) where it exceeds 0.5
+    float dmin = INFINITY, rmin = INFINITY;
     unsigned n_in = 0, bad = 0;
     bool two = false;
     __device__ __forceinline__ void node(float dv, float x, float y, float z, float drop, bool two_, bool finite) {
@@ -131,8 +132,9 @@ struct Sums<false> {  // FP32 values
         rmin = fminf(rmin, rho);
         if (!finite) bad = 1;
     }
-    // Sums of the warp, in lane 0.
-    __device__ __forceinline__ Part row() {
+    // Sums of the warp, in lane 0; false (in every lane) where one is not finite: a partial
+    // sum beyond FP32's range, or data that is not finite.  They then have to be formed in FP64.
+    __device__ __forceinline__ bool row(Part& p) {
         double n = 0.0;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
@@ -147,17 +149,17 @@ struct Sums<false> {  // FP32 values
             bad |= __shfl_down_sync(0xffffffffu, bad, off);
         }
         n = (double)__reduce_add_sync(0xffffffffu, n_in);
-        Part p;
         p.v[0] = d.value();
         p.v[1] = jx.value();
         p.v[2] = jy.value();
         p.v[3] = jz.value();
         p.v[4] = in.value() + (two ? 0.0 : n);
         p.v[5] = n;
-        p.v[6] = fmin(dmin == FLT_MAX ? DBL_MAX : 1.0 + (double)dmin, rmin == FLT_MAX ? DBL_MAX : (double)rmin);
+        p.v[6] = fmin(dmin == INFINITY ? DBL_MAX : 1.0 + (double)dmin, rmin == INFINITY ? DBL_MAX : (double)rmin);
         p.v[7] = (double)bad;
         p.v[8] = all.value();
-        return p;
+        const bool held = isfinite(d.h) && isfinite(jx.h) && isfinite(jy.h) && isfinite(jz.h) && isfinite(in.h) && isfinite(all.h);
+        return __shfl_sync(0xffffffffu, held, 0);
     }
 };
 
@@ -165,11 +167,21 @@ struct Sums<false> {  // FP32 values
 // nodes where it exceeds 0.5, their count, min rho, non-finite flag, sum rho1).
 // The droplet density is rho for one component and rho1 for two (state
 // rho1, d, j, A; rho2 = 1 + d - rho1 is recovered from the sums).
-template <bool WIDE>
-__device__ __forceinline__ void write_row(Sums<WIDE>& s, bool two, double* __restrict__ row) {
+// walk(sums) adds the thread's nodes.
+template <bool WIDE, class Walk>
+__device__ __forceinline__ void write_row(Walk walk, bool two, double* __restrict__ row) {
     __shared__ double sh[kDiagThreads / 32][kRow];
-    if constexpr (!WIDE) s.two = two;  // a thread without nodes takes part in the same shuffles
-    const Part p = s.row();
+    Part p;
+    {
+        Sums<WIDE> s;
+        walk(s);
+        if constexpr (!WIDE) s.two = two;  // a thread without nodes takes part in the same shuffles
+        if (!s.row(p)) {
+            Sums<true> w;
+            walk(w);
+            w.row(p);
+        }
+    }
     if ((threadIdx.x & 31) == 0)
         for (int k = 0; k < kRow; ++k) sh[threadIdx.x >> 5][k] = p.v[k];
     __syncthreads();
@@ -185,37 +197,37 @@ template <class T, int NC>
 __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(const T* __restrict__ m, Layout L,
                                                                double* __restrict__ rows) {
     constexpr bool WIDE = std::is_same<T, double>::value;
-    using V = typename std::conditional<WIDE, double, float>::type;
     using FM = FieldMap<T, 9 + NC>;
-    Sums<WIDE> s;
     const size_t N = (size_t)L.nx * L.ny * L.nz, F = L.fs;
-    for (size_t n = blockIdx.x * (size_t)kDiagThreads + threadIdx.x; n < N; n += (size_t)gridDim.x * kDiagThreads) {
-        size_t r;
-        int x, y, z;
-        if ((N >> 32) == 0) {  // 32-bit divisions when the box allows
-            const unsigned q = (unsigned)n / (unsigned)L.nx;
-            x = (int)((unsigned)n - q * (unsigned)L.nx);
-            z = (int)(q / (unsigned)L.ny);
-            y = (int)(q - (unsigned)z * (unsigned)L.ny);
-        } else {
-            x = (int)(n % L.nx);
-            r = n / L.nx;
-            y = (int)(r % L.ny);
-            z = (int)(r / L.ny);
-        }
-        const size_t i = L.at(x, y, z);
-        V v[9 + NC];
-        bool finite = true;
+    auto walk = [&](auto& s) {
+        using V = typename std::conditional<std::is_same<decltype(s), Sums<true>&>::value, double, float>::type;
+        for (size_t n = blockIdx.x * (size_t)kDiagThreads + threadIdx.x; n < N; n += (size_t)gridDim.x * kDiagThreads) {
+            int x, y, z;
+            if ((N >> 32) == 0) {  // 32-bit divisions when the box allows
+                const unsigned q = (unsigned)n / (unsigned)L.nx;
+                x = (int)((unsigned)n - q * (unsigned)L.nx);
+                z = (int)(q / (unsigned)L.ny);
+                y = (int)(q - (unsigned)z * (unsigned)L.ny);
+            } else {
+                x = (int)(n % L.nx);
+                const size_t r = n / L.nx;
+                y = (int)(r % L.ny);
+                z = (int)(r / L.ny);
+            }
+            const size_t i = L.at(x, y, z);
+            V v[9 + NC];
+            bool finite = true;
 #pragma unroll
-        for (int f = 0; f < 9 + NC; ++f) {
-            const T t = __ldg(m + FM::at(i, f, F));
-            if constexpr (IsNarrow<T>::value) v[f] = cv_field<V>(t, f);
-            else v[f] = (V)t;
-            finite = finite && isfinite(v[f]);
+            for (int f = 0; f < 9 + NC; ++f) {
+                const T t = __ldg(m + FM::at(i, f, F));
+                if constexpr (IsNarrow<T>::value) v[f] = cv_field<V>(t, f);
+                else v[f] = (V)t;
+                finite = finite && isfinite(v[f]);
+            }
+            s.node(v[NC - 1], v[NC], v[NC + 1], v[NC + 2], NC == 2 ? v[0] : V(1) + v[0], NC == 2, finite);
         }
-        s.node(v[NC - 1], v[NC], v[NC + 1], v[NC + 2], NC == 2 ? v[0] : V(1) + v[0], NC == 2, finite);
-    }
-    write_row(s, NC == 2, rows + (size_t)blockIdx.x * kRow);
+    };
+    write_row<WIDE>(walk, NC == 2, rows + (size_t)blockIdx.x * kRow);
 }
 
 // Sum of the rows, in a fixed order.
@@ -333,20 +345,21 @@ template <class T>
 __global__ void __launch_bounds__(kDiagThreads) k_diag_partial_canonical(const T* __restrict__ m, size_t N,
                                                                          double* __restrict__ rows) {
     constexpr bool WIDE = std::is_same<T, double>::value;
-    Sums<WIDE> s;
     const size_t lo = (size_t)blockIdx.x * kStaticNodesPerRow;
     const size_t hi = lo + kStaticNodesPerRow < N ? lo + kStaticNodesPerRow : N;
-    for (size_t i = lo + threadIdx.x; i < hi; i += kDiagThreads) {
-        T v[10];
-        bool finite = true;
+    auto walk = [&](auto& s) {
+        for (size_t i = lo + threadIdx.x; i < hi; i += kDiagThreads) {
+            T v[10];
+            bool finite = true;
 #pragma unroll
-        for (int f = 0; f < 10; ++f) {
-            v[f] = __ldg(m + f * N + i);
-            finite = finite && isfinite(v[f]);
+            for (int f = 0; f < 10; ++f) {
+                v[f] = __ldg(m + f * N + i);
+                finite = finite && isfinite(v[f]);
+            }
+            s.canonical(v[0], v[1], v[2], v[3], finite);
         }
-        s.canonical(v[0], v[1], v[2], v[3], finite);
-    }
-    write_row(s, false, rows + (size_t)blockIdx.x * kRow);
+    };
+    write_row<WIDE>(walk, false, rows + (size_t)blockIdx.x * kRow);
 }
 
 constexpr int kMaxDevices = 64;

@@ -36,6 +36,36 @@ struct Two {
     }
 };
 
+// A sum carried as h + l + m: h and l stay a renormalised pair, m collects what their
+// additions round off.  After n terms the error is at most about n^2 2^-75 of the largest
+// partial sum; FP64 has n 2^-53, more than that up to n = 2^22.  Exact but for that while
+// nothing overflows: check h, which stays infinite or NaN once a step of it was.
+struct Sum3 {
+    float h = 0.0f, l = 0.0f, m = 0.0f;
+
+    __device__ __forceinline__ void add(float a) {
+        const Two s = Two::sum(h, a), t = Two::sum(l, s.l);
+        m = __fadd_rn(m, t.l);
+        const Two r = Two::sum(s.h, t.h);
+        h = r.h;
+        l = r.l;
+    }
+    __device__ __forceinline__ void add(const Two& a) {
+        add(a.h);
+        add(a.l);
+    }
+    __device__ __forceinline__ void add(const Sum3& o) {
+        add(o.h);
+        add(o.l);
+        m = __fadd_rn(m, o.m);
+    }
+    __device__ __forceinline__ double value() const { return (double)h + ((double)l + (double)m); }
+    __device__ __forceinline__ Sum3 shfl_down(int off) const {
+        return {__shfl_down_sync(0xffffffffu, h, off), __shfl_down_sync(0xffffffffu, l, off),
+                __shfl_down_sync(0xffffffffu, m, off)};
+    }
+};
+
 // a + b + c rounded once: b + c and a + (b + c) as exact pairs, their low parts added with
 // rounding to odd, which keeps the last addition from rounding a second time (Boldo and
 // Melquiond, "Emulation of a FMA and correctly rounded sums", 2008).
