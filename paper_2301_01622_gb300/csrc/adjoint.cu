@@ -38,56 +38,25 @@
 #include <cmath>
 #include <vector>
 
+#include "adjoint_terms.cuh"
 #include "checked.cuh"
 #include "internal.h"
 #include "lattice.cuh"
 #include "layout.cuh"
 #include "moment_common.cuh"
 #include "moment_pair.cuh"
-#include "twofloat.cuh"
 
 namespace llb {
 namespace {
 
 constexpr int kAdjThreads = 128;
 
-// dL/domega term of a node, lam'_A : (j j / rho - A), and its sums.  In FP64 these
-// some 40 operations per node filled the FP64 pipe (two FMA per clock and SM; 79 %
-// busy) and set the time of the adjoint step, 62 of 62 us on 128 x 96 x 64 D3Q19
-// FP32.  For an FP32 state they run on pairs of FP32 numbers (twofloat.cuh); FP64
-// states keep FP64.
-template <class T>
-struct Wide;
-
-template <>
-struct Wide<double> {
-    double v = 0.0;
-    // += a (b r - c)
-    __device__ __forceinline__ void add_term(double a, double b, double r, double c) { v += a * (b * r - c); }
-    __device__ __forceinline__ double value() const { return v; }
-    __device__ __forceinline__ Wide shfl_down(int off) const { return {__shfl_down_sync(0xffffffffu, v, off)}; }
-    __device__ __forceinline__ void merge(const Wide& o) { v += o.v; }
-};
-
-template <>
-struct Wide<float> {
-    Two v;
-    __device__ __forceinline__ void add_term(float a, float b, float r, float c) {
-        const Two p = Two::prod(b, r), s = Two::sum(p.h, -c), x = Two::prod(a, s.h);
-        v.add(x.h);
-        v.l = __fadd_rn(v.l, __fmaf_rn(a, __fadd_rn(p.l, s.l), x.l));
-    }
-    __device__ __forceinline__ double value() const { return v.value(); }
-    __device__ __forceinline__ Wide shfl_down(int off) const { return {v.shfl_down(off)}; }
-    __device__ __forceinline__ void merge(const Wide& o) { v.add(o.v); }
-};
-
 // Sum of the block's terms, added to its row (fixed order: warp shuffles, then the warps).
 template <int NT, class T>
-__device__ __forceinline__ void add_block_sum(Wide<T> part, double* __restrict__ row) {
-    for (int off = 16; off > 0; off >>= 1) part.merge(part.shfl_down(off));
+__device__ __forceinline__ void add_block_sum(const Wide<T>& part, double* __restrict__ row) {
     __shared__ double wsum[NT / 32];
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = part.value();
+    const double own = part.warp_sum();
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = own;
     __syncthreads();
     if (threadIdx.x == 0) {
         double sacc = 0.0;
@@ -164,7 +133,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_step(const T* __restric
 #pragma unroll
         for (int f = 0; f < 10; ++f) lam[FieldMap<T, 10>::at(i0, f, lay.fs)] = out[f];
         // dL/domega: lam'_A : (j j / rho - A)
-        for (int k = 0; k < 6; ++k) part.add_term(la[k], jj[k], rinv, s[4 + k]);
+        part.add_node(la, jj, rinv, s + 4);
     }
     add_block_sum<kAdjThreads>(part, domega_rows + ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
@@ -183,26 +152,9 @@ struct Adjoint {
     float om;
     double* rows;
 
-    struct Sum {  // of the thread's two nodes, on pairs of FP32 numbers (as Wide<float>)
-        float2 h = {0.0f, 0.0f}, l = {0.0f, 0.0f};
+    struct Sum : PairSums {  // of the thread's two nodes (and wide_slot)
+        __device__ __forceinline__ Sum() { wide_slot() = 0.0; }
     };
-    // h + l += a, exactly but for the rounding of l
-    static __device__ __forceinline__ void add2(Sum& t, float2 a) {
-        using namespace pk;
-        const float2 s = pk::add(t.h, a), b = sub(s, t.h);
-        t.l = pk::add(t.l, pk::add(sub(t.h, sub(s, b)), sub(a, b)));
-        t.h = s;
-    }
-    // += a (b r - c)
-    static __device__ __forceinline__ void add_term(Sum& t, float2 a, float2 b, float2 r, float2 c) {
-        using namespace pk;
-        const float2 ph = mul(b, r), pl = fma(b, r, mul(-1.0f, ph));
-        Sum s{ph, pl};
-        add2(s, mul(-1.0f, c));
-        const float2 xh = mul(a, s.h), xl = fma(a, s.h, mul(-1.0f, xh));
-        add2(t, xh);
-        t.l = pk::add(t.l, fma(a, s.l, xl));
-    }
 
     __device__ __forceinline__ pk::Col<float2> column(const float2* v) const {
         using namespace pk;
@@ -246,6 +198,37 @@ struct Adjoint {
         const float2 rinv = fma(r0, sub(one, mul(r0, pk::add(one, s[0]))), r0);
         const float2 jx = s[1], jy = s[2], jz = s[3];
         const float2 jj[6] = {mul(jx, jx), mul(jy, jy), mul(jz, jz), mul(jx, jy), mul(jx, jz), mul(jy, jz)};
+        // dL/domega: lam'_A : (j j / rho - A) of the nodes inside the box
+        const bool ok[2] = {ok_lo, ok_hi};
+        bool held = true;
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            float ta[6], tb[6], tc[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                ta[k] = n ? la[k].y : la[k].x;
+                tb[k] = n ? jj[k].y : jj[k].x;
+                tc[k] = n ? s[4 + k].y : s[4 + k].x;
+            }
+            held = held && TermSizes(ta, tb, n ? rinv.y : rinv.x, tc).held();
+        }
+        if (held) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                total.add_terms(make_float2(ok_lo ? la[k].x : 0.0f, ok_hi ? la[k].y : 0.0f), jj[k], rinv, s[4 + k]);
+            total.renormalise();
+        } else {
+            // in FP64 and inline: the call of scaled_sum would spill registers (44 us a step, so 37,
+            // launched alone)
+            double w = 0.0;
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+                if (ok[n])
+                    for (int k = 0; k < 6; ++k)
+                        w += (double)(n ? la[k].y : la[k].x) *
+                             ((double)(n ? jj[k].y : jj[k].x) * (double)(n ? rinv.y : rinv.x) - (double)(n ? s[4 + k].y : s[4 + k].x));
+            wide_slot() += w;
+        }
         float2 dsum = mul(la[0], jj[0]);
 #pragma unroll
         for (int k = 1; k < 6; ++k) dsum = fma(la[k], jj[k], dsum);
@@ -257,19 +240,13 @@ struct Adjoint {
         r[3] = fma(-3.0f, q[3], mul(o, fma(jz2, la[2], fma(jx, la[4], mul(jy, la[5])))));
 #pragma unroll
         for (int k = 0; k < 6; ++k) r[4 + k] = mul(1.0f - om, la[k]);
-        // dL/domega: lam'_A : (j j / rho - A)
-        Sum t;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) add_term(t, la[k], jj[k], rinv, s[4 + k]);
-        if (!ok_lo) t.h.x = t.l.x = 0.0f;
-        if (!ok_hi) t.h.y = t.l.y = 0.0f;
-        add2(total, t.h);
-        total.l = pk::add(total.l, t.l);
     }
     __device__ __forceinline__ void end(const Sum& total) const {
-        Wide<float> part;
-        part.v = Two{total.h.x, total.l.x};
-        part.v.add(Two{total.h.y, total.l.y});
+        const double wide = wide_slot();
+        Wide<float> part;  // (clears the slot)
+        wide_slot() = wide;
+        part.v = total;
+        static_assert(mom::PairTile<L, mom::kPairH>::NT <= kWideThreads, "a slot per thread");
         add_block_sum<mom::PairTile<L, mom::kPairH>::NT>(part, rows + blockIdx.x);
     }
 };
@@ -411,7 +388,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_cg_local(const T* __res
         for (int f = 0; f < 11; ++f) lam[f * fs + i0] = out[f];
 #pragma unroll
         for (int a = 0; a < 3; ++a) lam_g[a * fs + i0] = lg[a];
-        for (int k = 0; k < 6; ++k) part.add_term(la[k], jj[k], rinv, A[k]);
+        part.add_node(la, jj, rinv, A);
     }
     add_block_sum<kAdjThreads>(part, domega_rows + ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
@@ -743,7 +720,7 @@ __device__ __forceinline__ void adj_receive(Wide<T>& part, const T* __restrict__
     for (int f = 0; f < 11; ++f) lam[f * fs + i0] = out[f];
 #pragma unroll
     for (int a = 0; a < 3; ++a) lam_g[a * fs + i0] = ln[a] * ign + l_gn * nv[a];
-    for (int k = 0; k < 6; ++k) part.add_term(la[k], jj[k], rinv, A[k]);
+    part.add_node(la, jj, rinv, A);
 }
 
 template <class L, class T, int BX, int BY>
