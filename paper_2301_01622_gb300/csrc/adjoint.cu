@@ -156,19 +156,22 @@ struct Adjoint {
         __device__ __forceinline__ Sum() { wide_slot() = 0.0; }
     };
 
+    // The sums of the pull are in units of the smallest weight w, up to 1 / w times their
+    // moments: the columns carry a power of two that keeps them in the range of those.
+    static constexpr float kDown = pk::Shells<L>::corners ? 0x1p-8f : 0x1p-6f;
     __device__ __forceinline__ pk::Col<float2> column(const float2* v) const {
         using namespace pk;
         Col<float2> c;
-        c.s = col_s(v[4], v[5], v[6], v[0]);
-        c.jx = mul(-1.0f, v[1]);
-        c.jy = mul(-1.0f, v[2]);
-        c.jz = mul(-1.0f, v[3]);
-        c.xx = v[4];
-        c.yy = v[5];
-        c.zz = v[6];
-        c.xy = v[7];
-        c.xz = v[8];
-        c.yz = v[9];
+        c.jx = mul(-kDown, v[1]);
+        c.jy = mul(-kDown, v[2]);
+        c.jz = mul(-kDown, v[3]);
+        c.xx = mul(kDown, v[4]);
+        c.yy = mul(kDown, v[5]);
+        c.zz = mul(kDown, v[6]);
+        c.xy = mul(kDown, v[7]);
+        c.xz = mul(kDown, v[8]);
+        c.yz = mul(kDown, v[9]);
+        c.s = col_s(c.xx, c.yy, c.zz, mul(kDown, v[0]));
         return c;
     }
     __device__ __forceinline__ void load(float* v, size_t e, size_t stride, size_t fs) const {
@@ -180,7 +183,8 @@ struct Adjoint {
     __device__ __forceinline__ void finish(float2* r, const float* a, const float* b, bool ok_lo, bool ok_hi,
                                            Sum& total) const {
         using namespace pk;
-        constexpr float wh = (float)Shells<L>::w, wl = (float)(Shells<L>::w - (double)wh);
+        constexpr double w = Shells<L>::w / kDown;
+        constexpr float wh = (float)w, wl = (float)(w - (double)wh);
         float2 q[10];
 #pragma unroll
         for (int f = 0; f < 10; ++f) q[f] = col_j(wh, wl, r[f]);

@@ -8,7 +8,9 @@ import numpy as np
 import pytest
 
 from paper_2301_01622_gb300 import build as B
+from paper_2301_01622_gb300 import inputs, llb
 
+torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -90,3 +92,29 @@ def test_terms_that_are_not_finite(sum_terms):
     assert sum_terms(a, b, r, c) == -np.inf
     c[40, 0] = np.nan
     assert np.isnan(sum_terms(a, b, r, c))
+
+
+@pytest.mark.parametrize("q", [19, 27])
+@pytest.mark.parametrize("ncomp", [1, 2])
+def test_dtau_beyond_the_range_of_float(ncomp, q):
+    """Finite cotangents whose terms add up to more than 3.4e38: against FP64 states, to the
+    1e-4 of the other FP32 gradients."""
+    shape = (40, 9, 6)
+    nf = 9 + ncomp
+    m = inputs.random_moments(*shape, seed=5, nfields=nf)
+    m[ncomp + 3:ncomp + 6] += 3.0  # A = 3, so every term is about as large as its cotangent
+    g = np.zeros_like(m)
+    g[ncomp + 3:ncomp + 6] = 3e36 * (1.0 + 0.1 * np.random.default_rng(1).normal(size=(3,) + m.shape[1:]))
+    res = []
+    for storage, dt in ((llb.LLB_F64, torch.float64), (llb.LLB_F32, torch.float32)):
+        gd = torch.from_numpy(g).to("cuda", dt)
+        gi = torch.empty_like(gd)
+        two = dict(ncomp=2, grad_eps=0.05) if ncomp == 2 else {}
+        c = llb.llb_create(*shape, q, 0.8, llb.llb_params_default(storage=storage, **two))
+        try:
+            llb.llb_init_moments(c, m)
+            res.append(llb.llb_adjoint(c, 1, gd, gi))
+        finally:
+            llb.llb_destroy(c)
+    assert abs(res[0]) > 3.5e38 and np.isfinite(res[1])
+    assert abs(res[1] - res[0]) <= 1e-4 * abs(res[0])
