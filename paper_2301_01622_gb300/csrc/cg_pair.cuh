@@ -38,7 +38,7 @@ namespace cg {
 // Constants of the scaled collision: w = the smallest weight.
 struct PairK {
     float ka, kc, ko;          // 4.5 w (1 - omega), 9 w (1 - omega), 4.5 w omega
-    float w, wj, wj2;          // w, 3 w and what rounding it left
+    float w, w2, wj, wj2;      // w and 3 w, each with what rounding it left
     float kg, bw, kf;          // 0.5 w A_s, beta w, 9 w (1 - omega / 2)
     float A_h, g_min, g_nci, eps2;
     int h_c;
@@ -52,6 +52,7 @@ PairK pair_constants(const llb_ctx& c) {
     k.kc = (float)(9.0 * w * (1.0 - om));
     k.ko = (float)(4.5 * w * om);
     k.w = (float)w;
+    k.w2 = (float)(w - (double)k.w);
     k.wj = (float)(3.0 * w);
     k.wj2 = (float)(3.0 * w - (double)k.wj);
     k.kg = (float)(0.5 * w * c.params.A_s);
@@ -131,7 +132,12 @@ __device__ __forceinline__ Src collide_pair(float2 r1, float2 d, const float2* m
     const float2 gn = mul(g2, ig);
     if (!(gn.x >= k.g_min)) ig.x = 0.0f;
     if (!(gn.y >= k.g_min)) ig.y = 0.0f;
-    const float2 rinv = rcp1p(1.0f, d);
+    // 1 / rho, refined: rho1 is carried by rho1 / rho and sums of it with the weights, so what
+    // the approximation or a weight is off by adds up from step to step (w2 for the same reason).
+    // Error of 384 x 192 x 192 D3Q27 droplets after 30 steps against 64 bits, 2-norm, six inputs:
+    // 3.6 to 6.2e-8 without the three, 2.3 to 3.2e-8 with them; 0.7 % of the step.
+    const float2 one = make_float2(1.0f, 1.0f), r0 = rcp1p(1.0f, d);
+    const float2 rinv = fma(r0, fma(sub(make_float2(-1.0f, -1.0f), d), r0, one), r0);
     Src s;
     s.r1 = mul(r1, rinv);
     // near-contact detector on the interface band
@@ -179,7 +185,7 @@ __device__ __forceinline__ Src collide_pair(float2 r1, float2 d, const float2* m
     }
     s.c.s = col_s(s.c.xx, s.c.yy, s.c.zz, mul(k.w, d));
     // e = beta rho1 rho2 / rho
-    const float2 rho2 = add(sub(make_float2(1.0f, 1.0f), r1), d);
+    const float2 rho2 = add(sub(one, r1), d);
     const float2 e = mul(mul(mul(k.bw, s.r1), rho2), ig);
     s.ex = mul(e, gx);
     s.ey = mul(e, gy);
@@ -435,9 +441,11 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
     auto row_copy = [&](int y) { return y < lay.yo ? ny * lay.px : y >= ny - lay.yo ? -ny * lay.px : 0; };
     const size_t o_lo = ok_lo ? lay.at(ox, oy, 0) : 0, o_hi = ok_hi ? lay.at(ox, oy + H, 0) : 0;
     // rolling sums of the plane ahead of the source plane (P) and of the source
-    // plane (A; zg, zx, zy: the c_z moments of its c_z = +1 pulls)
+    // plane (A; zg, zx, zy: the c_z moments of its c_z = +1 pulls).  Those of rho1 (Ph; Ah, Bh:
+    // c_z = 0 and +1) stay apart until the last plane: rho1 is of order one and two roundings at
+    // that size in every step, always the same way where the fluid is uniform, showed
     PlaneSum<float2> P{zero, zero, zero, zero, zero, zero}, A{zero, zero, zero, zero, zero, zero};
-    float2 zg = zero, zx = zero, zy = zero, Ph = zero, Ah = zero;
+    float2 zg = zero, zx = zero, zy = zero, Ph = zero, Ah = zero, Bh = zero;
 
 #pragma unroll 1
     for (int s = za - 4;; ++s) {
@@ -538,7 +546,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
             float2 ht = fma(l.r, l.t, fma(r.r, r.t, fma(u.r, u.t, mul(d.r, d.t))));
             float2 hc = fma(l.r, l.c1, fma(r.r, r.c1, fma(u.r, u.c1, mul(d.r, d.c1))));
             {
-                const float2 R = mul(k.w, add(add(l.r, r.r), add(u.r, d.r)));
+                const float2 R = col_j(k.w, k.w2, add(add(l.r, r.r), add(u.r, d.r)));
                 const float2 T = add(sub(lo2(B2[nl]), lo2(B2[nr])), sub(hi2(B2[nu]), hi2(B2[nd])));
                 const float2 Z = add(add(BZ[nl], BZ[nr]), add(BZ[nu], BZ[nd]));
                 h0 = mul(a0, add(h0, add(R, T)));
@@ -552,7 +560,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
                                      sub(add(hi2(e), hi2(f)), add(hi2(g), hi2(h))));
                 if constexpr (kC) {
                     const Nb pp = nb(4, nul), mm = nb(5, ndr), pm = nb(6, ndl), mp = nb(7, nur);
-                    const float2 R = mul(k.w, add(add(pp.r, mm.r), add(pm.r, mp.r)));
+                    const float2 R = col_j(k.w, k.w2, add(add(pp.r, mm.r), add(pm.r, mp.r)));
                     const float2 Z = add(add(BZ[nul], BZ[nur]), add(BZ[ndl], BZ[ndr]));
                     h0 = fma(pp.r, pp.c0, fma(mm.r, mm.c0, fma(pm.r, pm.c0, fma(mp.r, mp.c0, h0))));
                     ht = fma(pp.r, pp.t, fma(mm.r, mm.t, fma(pm.r, pm.t, fma(mp.r, mp.t, ht))));
@@ -566,7 +574,7 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
                 } else {
                     const float2 pp = G2[nul], mm = G2[HN + ndr], pm = G2[2 * HN + ndl], mp = G2[3 * HN + nur];
                     const float2 rp = lo2(B1[nul]), rm = lo2(B1[ndr]), rq = lo2(B1[ndl]), rs = lo2(B1[nur]);
-                    const float2 R = mul(k.w, add(add(rp, rm), add(rq, rs)));
+                    const float2 R = col_j(k.w, k.w2, add(add(rp, rm), add(rq, rs)));
                     h0 = fma(rp, pp, fma(rm, mm, fma(rq, pm, fma(rs, mp, h0))));
                     h0 = add(h0, fma(i2, T, R));
                     qt = plane_sum<false>(o1, a1, 1.0f, add(own_s, hi2(B1[n1])), l.t, r.t, u.t, d.t, zero, zero, zero, zero);
@@ -577,15 +585,16 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
             {  // own column
                 const float4 v = B1[n1];
                 const float2 rr = lo2(v), ws = add(own_s, make_float2(k.w, k.w));
-                h0 = fma(mul(o0, rr), ws, h0);
-                ht = fma(mul(o1, rr), add(ws, hi2(v)), ht);
+                const float2 r0 = mul(o0, rr), r1 = mul(o1, rr);
+                h0 = fma(r0, ws, fma(k.w2, r0, h0));
+                ht = fma(r1, add(ws, hi2(v)), fma(k.w2, r1, ht));
                 hc = fma(o1, fma(rr, own_z, BZ[n1]), hc);
             }
             {  // plane s - 1 is complete with the c_z = -1 pulls, qt - qc
                 float2 v[11];
                 const float third = (float)kCs2;
                 const float2 g = sub(qt.g, qc.g), jx = sub(qt.jx, qc.jx), jy = sub(qt.jy, qc.jy);
-                v[0] = add(Ah, sub(ht, hc));
+                v[0] = fma(s0, Ah, add(Bh, sub(ht, hc)));
                 v[1] = add(A.g, g);
                 v[2] = add(A.jx, jx);
                 v[3] = add(A.jy, jy);
@@ -655,7 +664,8 @@ __device__ __forceinline__ void cg_pair_item(const float* in, float* out, const 
             A.xx = fma(s0, q0.xx, P.xx);
             A.yy = fma(s0, q0.yy, P.yy);
             A.xy = kC ? fma(s0, q0.xy, P.xy) : q0.xy;
-            Ah = fma(s0, h0, Ph);
+            Ah = h0;
+            Bh = Ph;
             P.g = add(qt.g, qc.g);
             P.jx = add(qt.jx, qc.jx);
             P.jy = add(qt.jy, qc.jy);
