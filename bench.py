@@ -667,7 +667,7 @@ def main():
     if rank != 0:
         return
     nodes = NX * NY * NZ
-    traffic = ncu_traffic("moment_tiled_d3q19_f32")
+    traffic = ncu_traffic("moment_pair_d3q19_f32")
     roof = {"bound": "hbm", "achieved": main_r["achieved_gbs"], "peak": peak, "unit": "GB/s",
             "frac": main_r["achieved_gbs"] / peak, "traffic": traffic,
             "frac_of_nominal_7900": main_r["achieved_gbs"] / 7900.0,

@@ -102,8 +102,9 @@ typedef struct llb_params {
                          tiled kernel 0..5 (0: two nodes per thread, tile
                          30x6; one node per thread, 64x4: TMA L2 prefetch,
                          IEEE 1/rho, then 64x8 and 32x8 tiles, 64x4 with a
-                         split-phase plane barrier), TMA kernel 0..2 (ring depth, tile); the other
-                         storage types have one shape per kernel.  Two
+                         split-phase plane barrier), TMA kernel 0..2 (ring
+                         depth, tile); the other storage types have one shape
+                         per kernel (16-bit: two nodes per thread).  Two
                          components, FP32: 0..5 (0: two nodes per thread,
                          tile 28x10, approximate FP32 quotients; one node per
                          thread: 64x4, 32x8, 32x16 with IEEE quotients; 32x8
@@ -234,12 +235,14 @@ LLB_API int llb_get_moments(llb_ctx* ctx, void* host_out, int host_dtype);
 /* Same into caller DEVICE memory, asynchronous. */
 LLB_API int llb_get_moments_device(llb_ctx* ctx, void* dev_out, int dtype);
 
-/* FP64 reductions of the current state (Sec. IV, Figs. 2, 5, 7 and mass /
- * momentum conservation).  Synchronises the stream. */
+/* Reductions of the current state (Sec. IV, Figs. 2, 5, 7 and mass / momentum
+ * conservation), in FP64; sums over FP32 and 16-bit states are formed in three
+ * floats per thread, which are at least as accurate, and in FP64 where those
+ * overflow.  Synchronises the stream. */
 LLB_API int llb_diagnostics(llb_ctx* ctx, llb_diag* out);
 
 /* Diagnostics of canonical one-component moments (rho, j, P; layout above)
- * that are already in DEVICE memory, with the same FP64 sums as
+ * that are already in DEVICE memory, with the same sums as
  * llb_diagnostics, for callers that cannot allocate device memory.  The
  * paper has no counterpart: this is a deployment convenience.
  *

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_step(const T* __restric
 // a = lam_A.  The sums of the pull are the moments sum w_i s_i (1, -c, c c), from which
 // r_i . s_i and J_C^T follow per node.  A thread holds two nodes; loading all ten fields
 // of 19 neighbours per node, as k_adjoint_step does, kept the load pipe busy: 128 x 96 x
-// 64 D3Q19 took 40.7 us a step, now 26.5.
+// 64 D3Q19 took 40.7 us a step, now about 31 (26.5 without the exact sums of dL/domega).
 template <class L>
 struct Adjoint {
     static constexpr bool kAdjoint = true;
@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(kPhiX * kPhiY) k_adjoint_cg_phi(const T* __res
 // its own fields, where it evaluated the node's populations and their cotangents
 // direction by direction (2160 instructions per node on D3Q27).  Twelve warps per SM
 // (the ring) leave the loads exposed, so each plane is loaded one plane ahead: 96^3
-// D3Q27 FP32 91 us a step before, 71 now (95 without the loads ahead).
+// D3Q27 FP32 91 us a step before, 71 so (95 without the loads ahead), about 82 with the
+// exact sums of dL/domega.
 template <class L, class T, int BX, int BY>
 struct AdjTile {
     static constexpr int NT = BX * BY, HX = BX + 2, HY = BY + 2, HN = HX * HY;

@@ -671,7 +671,7 @@ struct CGShape {
     static constexpr bool PAIR = false;
 };
 // FP32, variant 0 (the default): two nodes per thread (cg_pair.cuh).  On the 384 x 192 x
-// 192 droplet pair 459 us per step on D3Q27 (30.8 k MLUPS) against 740 us of the best
+// 192 droplet pair 464 us per step on D3Q27 (30.5 k MLUPS) against 740 us of the best
 // one-node shape, 32 x 8 approximate rolled, whose place it takes.
 struct CGPair {
     static constexpr bool PAIR = true;

@@ -761,7 +761,8 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
 
 // Tiles of 28 x 10, two CTAs of six warps per SM (168 registers, no spills; 113 KB
 // of shared memory each on D3Q27).  Measured on 384 x 192 x 192 D3Q27 with a droplet
-// pair, 128^3 D3Q19 and 96^3 D3Q27 (A_h = 0): 459, 87, 45 us per step; one CTA of 12
+// pair, 128^3 D3Q19 and 96^3 D3Q27 (A_h = 0): 459, 87, 45 us per step (464 on the first since
+// the roundings of rho1 are kept small); one CTA of 12
 // warps (28 x 22): 463, 92, 49 us; CTAs of four warps (28 x 6): 531, 86, 53 us; eight
 // warps at 128 registers spill and lose 15 % and more.
 constexpr int kPairH = 5, kPairCtas = 2;

@@ -4,7 +4,7 @@
 // The march of moment_tiled.cuh with the work of a thread doubled.  The one-node
 // form executed 334 thread-instructions per node on D3Q19 at half the issue rate,
 // with 4.4 of 8 warps colliding a halo node per plane; the pair executes
-// 202 and a CTA's halo is one warp.
+// 219 and a CTA's halo is one warp.
 //
 // A CTA is H tile warps and a halo warp for the rows above and below.  A warp
 // holds 32 columns, the inner 30 its outputs: the outer two are collided for
@@ -428,11 +428,11 @@ __global__ void __launch_bounds__(32 * (H + 1), MINB)
     }
 }
 
-// Tiles of 30 x 6, four CTAs of four warps per SM (127 registers at most, no spills).
-// Measured without / with ghost copies, us per step: 256^3 D3Q19 267 / 277, D3Q27 290 /
+// Tiles of 30 x 6, four CTAs of four warps per SM (128 registers at most, no spills).
+// Measured without / with ghost copies, us per step, launched without overlap: 256^3 D3Q19 267 / 277, D3Q27 290 /
 // 303; 192^3 D3Q19 FP16 113 / 127; 131 x 97 x 75 D3Q27 24.6 / 28.7 (one node per
 // thread, with them in every step: 305, 342, 137, 35).  Two CTAs of eight warps (30 x 14):
-// 263 / 283, 300 / 324, 111 / 141, 26.8 / 32.8.
+// 263 / 283, 300 / 324, 111 / 141, 26.8 / 32.8.  Overlapped and without: 267, 288, 109, 22.2.
 constexpr int kPairH = 3, kPairCtas = 4;
 
 // Chunk length of a box whose items go through the queue.  Without ghost copies all

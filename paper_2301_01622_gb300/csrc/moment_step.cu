@@ -1,12 +1,14 @@
 // Moment-only lattice Boltzmann step, one component (Sec. II-III A): the
-// direct kernel and the dispatch of the three kernels.
+// direct kernel and the dispatch of the four kernels.
 //
 //   * k_moment_direct: one thread per output node, gathers the ten moments of
 //     each of its Q neighbours and repeats the collision per neighbour.
 //     Shape-agnostic; the reference GPU path.
-//   * k_moment_tiled (moment_tiled.cuh, one translation unit per storage
-//     type): persistent z-marching kernel with plain loads and a TMA L2
-//     prefetch of the planes ahead; the default.
+//   * k_moment_pair (moment_pair.cuh): persistent z-marching kernel, two nodes per
+//     thread; the default for FP32 arithmetic.
+//   * k_moment_tiled (moment_tiled.cuh, one translation unit per storage type): the
+//     same march with one node per thread, plain loads and, in one variant, a TMA
+//     L2 prefetch of the planes ahead; the default for FP64, variants 1 to 5 of FP32.
 //   * k_moment_tma (moment_tma.cu): the same march with the planes staged in
 //     shared memory by TMA box loads.
 #include <cuda_runtime.h>

@@ -245,10 +245,10 @@ struct TiledShape {
     static constexpr int BX = BX_, BY = BY_, MINB = MINB_, OPT = OPT_, PD = PD_;
 };
 
-// FP32 variants 1-5 (variant 0 runs two nodes per thread: faster at every size
-// measured, D3Q19 steps of a graph, us: 16^3 3.3 against 3.7 of <64, 4, 2>, 32^3 4.55 /
-// 5.0, 64^3 8.9 / 9.6, 80^3 11.6 / 19.2, 128^3 41 / 48.6, 256^3 267 / 305; D3Q27 32^3
-// 5.5 / 5.6, 64^3 11.0 / 10.9, 80^3 14.2 / 22.2).  The approximate 1/rho is used by all
+// FP32 variants 1-5 (variant 0 runs two nodes per thread, faster than <64, 4, 2> at all
+// sizes measured but one; D3Q19 steps of a graph, us: 16^3 3.3 against 3.7, 32^3 4.55 / 5.0,
+// 64^3 8.9 / 9.6, 80^3 11.6 / 19.2, 128^3 41 / 48.6, 256^3 267 / 305; D3Q27 32^3 5.5 / 5.6,
+// 64^3 11.0 / 10.9, 80^3 14.2 / 22.2).  The approximate 1/rho is used by all
 // but variant 2 (measured ~1.5 % faster at 256^3, error far below FP32 storage
 // rounding).  The L2 prefetch (variant 1) measured 5 % slower than plain
 // loads on GB300 and is kept for the autotuner.

@@ -1,20 +1,22 @@
 // Step kernels launched one after the other on a stream, each set up while the CTAs of
 // the one before it end (programmatic dependent launch).  It saves the launch between
 // two short steps: 50 steps with their conversions, launched by llb_step, of 131 x 97 x
-// 75 D3Q27 1267 to 1142 us, of two components at 128^3 D3Q19 with diagnostics 4471 to
-// 4357; the replayed graph of 200 steps of 32^3 925 to 884.
+// 75 D3Q27 1269 to 1161 us, of two components at 128^3 D3Q19 with diagnostics 4512 to
+// 4400; the replayed graph of 200 steps of 32^3 955 to 917.
 //
 // A kernel launched with launch_overlapped may start once every CTA of the kernel
 // before it has called dep_launch (or has ended); it touches no global memory before
 // dep_wait, which returns when the kernel before it has ended and its writes are
 // visible.  dep_launch comes when a CTA has no item left: called at the start, the
 // waiting CTAs of the next step take the place of running ones (graph steps of 48^3
-// 6.4 us, so 5.6, without overlap 5.8; 32^3 5.0, 4.55, 4.75).  After a kernel that never calls dep_launch, or a copy, the launch is an ordinary one.
+// 6.4 us, so 5.6, without overlap 5.8; 32^3 5.05, 4.6, 4.8).  After a kernel that never
+// calls dep_launch, or a copy, the launch is an ordinary one.
 //
 // What the kernel before wrote is read with load_dep and through pointers that are not
 // __restrict__.  The non-coherent load (__ldg, or what the compiler makes of a const
 // __restrict__ pointer) is for data that is read-only for the whole life of a kernel, and
-// the life of these begins while the kernel before still writes.
+// the life of these begins while the kernel before still writes.  It was faster (256^3 D3Q19
+// 1 %, 200 steps of 32^3 in a graph 884 us against 917).
 #pragma once
 
 #include <cuda_runtime.h>

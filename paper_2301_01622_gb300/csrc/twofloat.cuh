@@ -1,12 +1,13 @@
-// Numbers carried as an unevaluated sum h + l of two floats (h rounded to nearest,
-// l the rounding error), for sums and differences that must not lose what FP64
-// would keep.  GB300's FP64 pipe does two FMA per clock and SM; kernels that read
-// FP32 and need a few more bits are several times faster on these.
-// Sums by Knuth's two-sum, products by FMA; relative error about 2^-46.
+// Numbers carried as unevaluated sums of floats, for sums, differences and quotients that
+// must not lose what FP64 would keep.  GB300's FP64 pipe does two FMA per clock and SM;
+// kernels that read FP32 and need more bits are several times faster on these.  Sums by
+// Knuth's two-sum, products by FMA: both exact while nothing overflows or, for products,
+// underflows.
 #pragma once
 
 namespace llb {
 
+// h + l, h rounded to nearest
 struct Two {
     float h = 0.0f, l = 0.0f;
 
@@ -19,20 +20,6 @@ struct Two {
     __device__ __forceinline__ static Two prod(float a, float b) {
         const float p = __fmul_rn(a, b);
         return {p, __fmaf_rn(a, b, -p)};
-    }
-    __device__ __forceinline__ void add(float a) {
-        const Two s = sum(h, a);
-        h = s.h;
-        l = __fadd_rn(l, s.l);
-    }
-    __device__ __forceinline__ void add(const Two& o) {
-        add(o.h);
-        l = __fadd_rn(l, o.l);
-    }
-    // an infinite or NaN sum is h alone: its rounding error is not a number
-    __device__ __forceinline__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
-    __device__ __forceinline__ Two shfl_down(int off) const {
-        return {__shfl_down_sync(0xffffffffu, h, off), __shfl_down_sync(0xffffffffu, l, off)};
     }
 };
 
