@@ -525,7 +525,7 @@ int llb_autotune(llb_ctx* c, int trials, int* kernel, int* variant) {
     drop_graphs(c);
     if (kernel) *kernel = c->kernel;
     if (variant) *variant = c->variant;
-    return LLB_OK;
+    return check_kernel_error(c);
 }
 
 int llb_get_moments(llb_ctx* c, void* host_out, int host_dtype) {

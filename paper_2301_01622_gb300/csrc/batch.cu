@@ -299,6 +299,20 @@ int llb_batch_autotune(llb_batch* b, int trials, int* variant) {
         return rc;
     }
     if (variant) *variant = win;
+    // the trials have been waited for: a wait that gave up in one of them is reported here
+    for (llb_ctx* c : b->ctx) {
+        int err = 0;
+        if (cudaMemcpyAsync(&err, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, b->stream) != cudaSuccess ||
+            cudaStreamSynchronize(b->stream) != cudaSuccess) {
+            cudaGetLastError();
+            b->sticky = LLB_ECUDA;
+            return LLB_ECUDA;
+        }
+        if (err) {
+            b->sticky = LLB_ETIMEOUT;
+            return LLB_ETIMEOUT;
+        }
+    }
     return LLB_OK;
 }
 

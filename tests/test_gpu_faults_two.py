@@ -102,3 +102,23 @@ def test_adjoint_reports_the_timeout(params):
     finally:
         llb.llb_destroy(ctx)
     _device_still_works()
+
+
+def test_autotuners_report_the_timeout():
+    """Their trials run the kernel that waits, and they synchronise."""
+    c = llb.llb_create(*SHAPE, 19, 0.9, llb.llb_params_default(**STUCK))
+    try:
+        llb.llb_init_moments(c, _drop(SHAPE))
+        assert _status(llb.llb_autotune, c, 1) == llb.LLB_ETIMEOUT
+        assert _status(llb.llb_step, c, 1) == llb.LLB_ESTATE
+    finally:
+        llb.llb_destroy(c)
+    b = llb.llb_batch_create([(8, 6, 5), (16, 9, 7)], 19, 0.9, llb.llb_params_default(**STUCK))
+    try:
+        for k, d in enumerate([(8, 6, 5), (16, 9, 7)]):
+            llb.llb_init_moments(llb.llb_batch_domain(b, k), _drop(d))
+        assert _status(llb.llb_batch_autotune, b, 1) == llb.LLB_ETIMEOUT
+        assert _status(llb.llb_batch_step, b, 1) == llb.LLB_ESTATE
+    finally:
+        llb.llb_batch_destroy(b)
+    _device_still_works()
