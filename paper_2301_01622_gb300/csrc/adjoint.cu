@@ -54,6 +54,7 @@ constexpr int kAdjThreads = 128;
 // Sum of the block's terms, added to its row (fixed order: warp shuffles, then the warps).
 template <int NT, class T>
 __device__ __forceinline__ void add_block_sum(const Wide<T>& part, double* __restrict__ row) {
+    static_assert(NT <= kWideThreads, "a slot per thread");
     __shared__ double wsum[NT / 32];
     const double own = part.warp_sum();
     if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = own;
@@ -250,7 +251,6 @@ struct Adjoint {
         Wide<float> part;  // (clears the slot)
         wide_slot() = wide;
         part.v = total;
-        static_assert(mom::PairTile<L, mom::kPairH>::NT <= kWideThreads, "a slot per thread");
         add_block_sum<mom::PairTile<L, mom::kPairH>::NT>(part, rows + blockIdx.x);
     }
 };
